@@ -1,5 +1,5 @@
 // lbm_host.cpp -- host FP64 helpers of liblbm: critical temperature, Maxwell
-// coexistence densities, parameter validation and built-in initial fields.
+// coexistence densities, parameter validation.
 #include "lbm_host.h"
 
 #include <cmath>
@@ -29,14 +29,6 @@ double bisect(F f, double lo, double hi, int iters = 200)
         if ((fm < 0) == (flo < 0)) { lo = mid; flo = fm; } else hi = mid;
     }
     return 0.5 * (lo + hi);
-}
-
-uint64_t splitmix64(uint64_t x)
-{
-    uint64_t z = x + 0x9E3779B97F4A7C15ull;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
 }
 
 bool finite_pos(double v) { return std::isfinite(v) && v > 0; }
@@ -202,33 +194,10 @@ int lbm_validate_params(const lbm_params* p)
     return LBM_OK;
 }
 
-int lbm_preset_field(int nx, int ny, int kind, double size, double width, double rho_l, double rho_v,
-                     int32_t cell, uint64_t seed, double noise_amp, std::vector<double>& out)
+int lbm_validate_preset(int nx, int ny, int kind, double size, double width, int32_t cell)
 {
     if (nx < 1 || ny < 1 || !(width > 0) || !std::isfinite(size)) return LBM_E_INVALID;
     if (kind < LBM_SLAB || kind > LBM_DROPLET_ARRAY) return LBM_E_INVALID;
     if (kind == LBM_DROPLET_ARRAY && cell < 1) return LBM_E_INVALID;
-    out.assign((size_t)nx * ny, 0.0);
-    for (int y = 0; y < ny; ++y)
-        for (int x = 0; x < nx; ++x) {
-            double d;
-            if (kind == LBM_SLAB) {
-                d = std::fabs(y - ny / 2.0) - size;
-            } else if (kind == LBM_DROPLET_ARRAY) {
-                const double cx = std::floor(double(x) / cell) * cell + cell / 2.0;
-                const double cy = std::floor(double(y) / cell) * cell + cell / 2.0;
-                d = std::hypot(x - cx, y - cy) - size;
-            } else {
-                d = std::hypot(x - nx / 2.0, y - ny / 2.0) - size;
-            }
-            const double inside = 0.5 * (1.0 - std::tanh(2.0 * d / width));
-            double r = (kind == LBM_BUBBLE) ? rho_l + (rho_v - rho_l) * inside : rho_v + (rho_l - rho_v) * inside;
-            if (noise_amp != 0.0) {
-                const uint64_t z = splitmix64(seed ^ (uint64_t)((size_t)y * nx + x));
-                const double xi = double(z >> 11) * (1.0 / 9007199254740992.0);
-                r += noise_amp * (2.0 * xi - 1.0);
-            }
-            out[(size_t)y * nx + x] = r;
-        }
     return LBM_OK;
 }

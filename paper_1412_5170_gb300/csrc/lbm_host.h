@@ -3,7 +3,6 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
-#include <vector>
 
 #include "lbm.h"
 // LBM_HOST_ARITHMETIC: the per-node arithmetic compiled by a host compiler
@@ -20,9 +19,8 @@ int lbm_maxwell(double T_over_Tc, double* rho_v, double* rho_l);
 // LBM_OK or LBM_E_INVALID / LBM_E_UNSUPPORTED for a parameter set.
 int lbm_validate_params(const lbm_params* p);
 
-// Initial density field of lbm_init_preset (row-major ny*nx).
-int lbm_preset_field(int nx, int ny, int kind, double size, double width, double rho_l, double rho_v,
-                     int32_t cell, uint64_t seed, double noise_amp, std::vector<double>& out);
+// LBM_OK or LBM_E_INVALID for the arguments of a built-in field (lbm_init_preset).
+int lbm_validate_preset(int nx, int ny, int kind, double size, double width, int32_t cell);
 
 // Polls of a bounded stage wait (mbarrier try_wait) before the staged kernels
 // declare a row copy stuck, flag a timeout, drain and return.
