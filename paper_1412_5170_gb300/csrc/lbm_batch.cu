@@ -20,6 +20,7 @@
 
 #include "lbm.h"
 #include "lbm_batch.cuh"
+#include "lbm_fields.cuh"
 #include "lbm_host.h"
 #include "lbm_warp.cuh"
 
@@ -309,27 +310,6 @@ k_reduce_batch(const BInst* __restrict__ inst, const BPart* __restrict__ parts, 
     }
 }
 
-__device__ __forceinline__ unsigned long long splitmix64_dev(unsigned long long x)
-{
-    unsigned long long z = x + 0x9E3779B97F4A7C15ull;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
-
-// Signed distance to the liquid of node (x, y) of an instance (slab, droplet,
-// bubble: distance to the gas region is returned negated by the caller).
-__device__ __forceinline__ double preset_distance(const BInst* I, int x, int y)
-{
-    if (I->kind == LBM_SLAB) return fabs(y - I->ny / 2.0) - I->size;
-    if (I->kind == LBM_DROPLET_ARRAY) {
-        const double cx = floor(double(x) / I->cell) * I->cell + I->cell / 2.0;
-        const double cy = floor(double(y) / I->cell) * I->cell + I->cell / 2.0;
-        return hypot(x - cx, y - cy) - I->size;
-    }
-    return hypot(x - I->nx / 2.0, y - I->ny / 2.0) - I->size;
-}
-
 // Grid of an instance's radial profile (mirrors lbm_profile_geom): sample k
 // at signed position centre + spacing (k - (nb - 1)/2) from the centre / mid-row.
 struct BGeom { int use, pad; double centre, spacing; };
@@ -353,34 +333,47 @@ __device__ __forceinline__ double profile_at(const double* p, int nb, const BGeo
     return p[k0] + t * (p[k0 + 1] - p[k0]);
 }
 
+// Walks a thread over the nodes of an nx-wide instance in steps of the grid's
+// threads, keeping (x, y) without a division per node.
+struct NodeWalk {
+    unsigned id, step;
+    int x, y, nx, sx, sy;
+    __device__ __forceinline__ explicit NodeWalk(int nx_)
+        : id(blockIdx.x * blockDim.x + threadIdx.x), step(gridDim.x * blockDim.x), nx(nx_)
+    {
+        y = int(id / unsigned(nx));
+        x = int(id - unsigned(y) * unsigned(nx));
+        sy = int(step / unsigned(nx));
+        sx = int(step - unsigned(sy) * unsigned(nx));
+    }
+    __device__ __forceinline__ void next()
+    {
+        id += step;
+        x += sx;
+        y += sy;
+        if (x >= nx) { x -= nx; ++y; }
+    }
+};
+
 // Initial density rho0 of every instance into the FP64 node array: its
 // preset (tanh profile plus SplitMix64 noise) or, where geom[i].use, its
-// radial profile.
-__global__ void k_rho0_batch(const BInst* __restrict__ inst, int n_inst, double* __restrict__ rho0,
-                             const double* __restrict__ prof, const BGeom* __restrict__ geom, int nb)
+// radial profile.  FP64-bound: see preset_density.
+__global__ void __launch_bounds__(256)
+k_rho0_batch(const BInst* __restrict__ inst, int n_inst, double* __restrict__ rho0, const double* __restrict__ prof,
+             const BGeom* __restrict__ geom, int nb)
 {
     const int i = blockIdx.y;
     if (i >= n_inst) return;
     const BInst* I = inst + i;
-    const int nx = I->nx, ny = I->ny;
-    const size_t n = (size_t)nx * ny;
-    const bool use_prof = prof && geom[i].use;
-    for (size_t id = blockIdx.x * (size_t)blockDim.x + threadIdx.x; id < n; id += (size_t)gridDim.x * blockDim.x) {
-        const int x = int(id % nx), y = int(id / nx);
-        double r;
-        if (use_prof) {
-            r = profile_at(prof + (size_t)i * nb, nb, geom[i], radial_distance(I, x, y));
-        } else {
-            const double d = preset_distance(I, x, y);
-            const double in = 0.5 * (1.0 - tanh(2.0 * d / I->width));
-            r = (I->kind == LBM_BUBBLE) ? I->rho_l + (I->rho_v - I->rho_l) * in
-                                        : I->rho_v + (I->rho_l - I->rho_v) * in;
-            if (I->noise_amp != 0.0) {
-                const unsigned long long z = splitmix64_dev(I->seed ^ (unsigned long long)((size_t)y * nx + x));
-                r += I->noise_amp * (2.0 * (double(z >> 11) * (1.0 / 9007199254740992.0)) - 1.0);
-            }
-        }
-        rho0[I->node_off + id] = r;
+    const unsigned n = unsigned(I->nx) * unsigned(I->ny);
+    double* out = rho0 + I->node_off;
+    if (prof && geom[i].use) {
+        for (NodeWalk w(I->nx); w.id < n; w.next())
+            out[w.id] = profile_at(prof + (size_t)i * nb, nb, geom[i], radial_distance(I, w.x, w.y));
+    } else {
+        const PresetField f{I->kind, I->nx, I->ny, I->cell, I->size, I->width, I->rho_l, I->rho_v, I->noise_amp, I->seed};
+        const double iw4 = 4.0 / f.width;
+        for (NodeWalk w(I->nx); w.id < n; w.next()) out[w.id] = preset_density(f, iw4, w.x, w.y);
     }
 }
 
@@ -420,33 +413,47 @@ __global__ void k_rest_velocity(const BInst* __restrict__ inst, int n_inst, cons
 // pull-convention FP32 deviations: the value stored at x for direction a is
 // the one that arrives at x + e_a, f_a = w_a rho0 (1 + 3 e.u + 9/2 (e.u)^2 -
 // 3/2 u.u) there (Eq. 2 with c_s^2 = 1/3), minus w_a rho_ref.
-__global__ void k_pops_batch(const BInst* __restrict__ inst, int n_inst, float* __restrict__ f,
-                             const double* __restrict__ rho0, const Snap* __restrict__ u0,
-                             const BGeom* __restrict__ geom)
+//
+// A thread takes the node whose populations it computes and writes each to
+// the node it is stored at, x - e_a (stores of a warp stay contiguous), so a
+// start from w rho0 needs its three distinct FP64 products once a node.
+// Gathered per stored node instead, with a 64-bit division each, the nine
+// products made this FP64-bound (5.6 ms for a sweep of 256 instances, 25 M
+// nodes).  With the fields of preset_density the whole lbm_batch_init of that
+// sweep went from 8.5 to 1.7 ms.
+__global__ void __launch_bounds__(256)
+k_pops_batch(const BInst* __restrict__ inst, int n_inst, float* __restrict__ f, const double* __restrict__ rho0,
+             const Snap* __restrict__ u0, const BGeom* __restrict__ geom)
 {
     const int i = blockIdx.y;
     if (i >= n_inst) return;
     const BInst* I = inst + i;
     const int nx = I->nx, ny = I->ny;
-    const size_t n = (size_t)nx * ny;
+    const unsigned n = unsigned(nx) * unsigned(ny);
     const double* r0 = rho0 + I->node_off;
-    const bool rest = u0 && geom && geom[i].use;
-    for (size_t id = blockIdx.x * (size_t)blockDim.x + threadIdx.x; id < n; id += (size_t)gridDim.x * blockDim.x) {
-        const int x = int(id % nx), y = int(id / nx);
+    const Snap* u = u0 && geom && geom[i].use ? u0 + I->node_off : nullptr;
+    const double ref = double(I->k.rho_ref);
+    float* fi = f + I->off;
+    for (NodeWalk w(nx); w.id < n; w.next()) {
+        const int xl = dec1(w.x, nx), xr = inc1(w.x, nx);
+        const size_t row = (size_t)w.y * nx, rd = (size_t)dec1(w.y, ny) * nx, ru = (size_t)inc1(w.y, ny) * nx;
+        const double r = r0[w.id];
+        double v[9];
 #pragma unroll
-        for (int a = 0; a < 9; ++a) {
-            const int xs = ex(a) > 0 ? inc1(x, nx) : (ex(a) < 0 ? dec1(x, nx) : x);
-            const int ys = ey(a) > 0 ? inc1(y, ny) : (ey(a) < 0 ? dec1(y, ny) : y);
-            const size_t src = (size_t)ys * nx + xs;
-            const double w = wt<double>(a), r = r0[src];
-            double v = w * r - w * double(I->k.rho_ref);
-            if (rest) {
-                const Snap u = u0[I->node_off + src];
-                const double ux = u.vx, uy = u.vy;
+        for (int a = 0; a < 9; ++a) v[a] = wt<double>(a) * r - wt<double>(a) * ref;
+        if (u) {
+            const Snap s = u[w.id];
+            const double ux = s.vx, uy = s.vy;
+#pragma unroll
+            for (int a = 0; a < 9; ++a) {
                 const double eu = ex(a) * ux + ey(a) * uy;
-                v += w * r * (3.0 * eu + 4.5 * eu * eu - 1.5 * (ux * ux + uy * uy));
+                v[a] += wt<double>(a) * r * (3.0 * eu + 4.5 * eu * eu - 1.5 * (ux * ux + uy * uy));
             }
-            f[I->off + a * n + id] = float(v);
+        }
+#pragma unroll
+        for (int a = 0; a < 9; ++a) {   // to (x, y) - e_a
+            const size_t at = (ey(a) > 0 ? rd : (ey(a) < 0 ? ru : row)) + (ex(a) > 0 ? xl : (ex(a) < 0 ? xr : w.x));
+            fi[(size_t)a * n + at] = float(v[a]);
         }
     }
 }

@@ -23,19 +23,20 @@ __device__ __forceinline__ unsigned long long splitmix64_dev(unsigned long long 
     return z ^ (z >> 31);
 }
 
-// rho0 of node (x, y): rho_v + (rho_l - rho_v) in + noise with
+// rho0 of node (x, y) (inv_width4 = 4 / width): rho_v + (rho_l - rho_v) in + noise with
 // in = (1 - tanh(2 d / width))/2 and d the signed distance to the liquid (a
 // bubble swaps the phases).
 //
-// Bound by the FP64 pipe, which is 1/60 of the FP32 one here: hypot, the
-// division and tanh are some 150 FP64 instructions, so they are evaluated
-// only where the result depends on them.
-//   - Centres are half-integers, so the squared distance (in units of 1/4) is
-//     an integer, and its correctly rounded root replaces hypot.
-//   - tanh(z) is 1 in FP64 from z = 19.1 on: where an FP32 estimate of the
-//     distance (good to 1e-6 of the lengths it is made of) puts the node more
-//     than ten widths (z = 20) from the interface, in is exactly 0 or 1.
-__device__ __forceinline__ double preset_density(const PresetField& f, int x, int y)
+// Bound by the FP64 pipe, which is 1/60 of the FP32 one here: hypot, two
+// divisions and tanh are some 150 FP64 instructions.  So
+//   - centres are half-integers, so the squared distance (in units of 1/4) is
+//     an integer, and its correctly rounded root replaces hypot;
+//   - (1 - tanh z)/2 = 1/(1 + exp(2z)), which also loses nothing to
+//     cancellation on the vapour side;
+//   - where an FP32 estimate of the distance (good to 1e-6 of the lengths it
+//     is made of) puts the node more than ten widths (z = 20) from the
+//     interface, in is 0 or 1 to 5e-18, and neither is evaluated.
+__device__ __forceinline__ double preset_density(const PresetField& f, double inv_width4, int x, int y)
 {
     unsigned long long q = 0;   // (2 distance)^2 to the centre; slab: 2 distance to the mid-row
     if (f.kind == LBM_SLAB) {
@@ -62,7 +63,7 @@ __device__ __forceinline__ double preset_density(const PresetField& f, int x, in
         in = 1.0;
     } else {
         const double r = f.kind == LBM_SLAB ? 0.5 * (double)q : 0.5 * sqrt((double)q);
-        in = 0.5 * (1.0 - tanh(2.0 * (r - f.size) / f.width));
+        in = 1.0 / (1.0 + exp((r - f.size) * inv_width4));
     }
     double rho = f.kind == LBM_BUBBLE ? f.rho_l + (f.rho_v - f.rho_l) * in : f.rho_v + (f.rho_l - f.rho_v) * in;
     if (f.noise_amp != 0.0) {
