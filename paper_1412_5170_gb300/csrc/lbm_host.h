@@ -39,40 +39,59 @@ int lbm_strip_launch(const lbm_params* p, int cfg, const void* fin, void* fout, 
                      long long first_wait = kStageWaitPolls);
 
 #if defined(__CUDACC__) || defined(LBM_HOST_ARITHMETIC)
-// Kernel constants of a parameter set in the compute type C.
+// Kernel constants of a parameter set in the compute type C: the FP32 path's
+// Coef<float>, or Coef<double>.
 template <typename C>
 lbm::Coef<C> make_coef(const lbm_params& p)
 {
     lbm::Coef<C> k;
-    k.T = C(p.T_over_Tc * lbm_tc());
-    k.K = C(p.K);
-    k.half_A = C(0.5 * p.A);
-    k.one_m_A = C(1.0 - p.A);
-    k.omega = C(1.0 / p.tau);
-    k.tau = C(p.tau);
-    k.guo_pre = C(1.0 - 0.5 / p.tau);
-    k.s_e = C(p.s_e);
-    k.s_eps = C(p.s_eps);
-    k.s_q = C(p.s_q);
-    k.rho_ref = C(p.precision == LBM_FP64 ? 0.0 : p.rho_ref);
-    k.li_c = C(p.forcing == LBM_LI ? p.sigma / (p.tau - 0.5) : 0.0);
-    const double rate[4] = {p.s_e, p.s_eps, p.s_q, 1.0 / p.tau};
-    const double norm[4] = {36.0, 36.0, 12.0, 4.0};
-    for (int i = 0; i < 4; ++i) {
-        k.r0[i] = C((1.0 - rate[i]) / norm[i]);
-        k.r1[i] = C(rate[i] / norm[i]);
-        k.r2[i] = C((1.0 - 0.5 * rate[i]) / norm[i]);
-    }
-    // FP32: omega and Guo's 1 - omega/2 both exact floats (omega moved by at
-    // most one ulp of 1 - omega/2 where needed), so that the momentum a step
-    // adds, omega F/2 + (1 - omega/2) F, is exactly F; the Shan-Chen shift
-    // tau = 1/omega as hi + lo.
-    k.A = C(p.A);
-    k.tau_lo = C(0);
-    k.h_e = C(1.0f - 0.5f * float(p.s_e));
-    k.h_eps = C(1.0f - 0.5f * float(p.s_eps));
-    k.h_q = C(1.0f - 0.5f * float(p.s_q));
-    if (p.precision != LBM_FP64) {
+    const double li_c = p.forcing == LBM_LI ? p.sigma / (p.tau - 0.5) : 0.0;
+    if constexpr (sizeof(C) == sizeof(double)) {
+        const double om = 1.0 / p.tau, pre = 1.0 - 0.5 / p.tau;
+        k.T = p.T_over_Tc * lbm_tc();
+        k.K2 = 2.0 * p.K;
+        k.half_A = 0.5 * p.A;
+        k.one_m_A = 1.0 - p.A;
+        k.omega = om;
+        k.one_m_omega = 1.0 - om;
+        k.tau = p.tau;
+        k.rho_ref = 0.0;
+        k.li_c = li_c;
+        k.w3 = 3.0 * om;
+        k.w45 = 4.5 * om;
+        k.g3 = 3.0 * pre;
+        k.g9 = 9.0 * pre;
+        k.e0 = (1.0 - p.s_e) / 36.0;
+        k.e1 = p.s_e / 12.0;
+        k.e2 = p.s_e / 18.0;
+        k.e3 = (1.0 - 0.5 * p.s_e) / 6.0;
+        k.p0 = (1.0 - p.s_eps) / 36.0;
+        k.p1 = p.s_eps / 36.0;
+        k.p2 = p.s_eps / 12.0;
+        k.p3 = (1.0 - 0.5 * p.s_eps) / 6.0;
+        k.q0 = (1.0 - p.s_q) / 12.0;
+        k.q1 = p.s_q / 12.0;
+        k.q2 = (1.0 - 0.5 * p.s_q) / 12.0;
+        k.n0 = (1.0 - om) / 4.0;
+        k.n1 = om / 4.0;
+        k.n2 = pre / 4.0;
+        return k;
+    } else {
+        k.T = C(p.T_over_Tc * lbm_tc());
+        k.K = C(p.K);
+        k.s_e = C(p.s_e);
+        k.s_eps = C(p.s_eps);
+        k.s_q = C(p.s_q);
+        k.rho_ref = C(p.rho_ref);
+        k.li_c = C(li_c);
+        // omega and Guo's 1 - omega/2 both exact floats (omega moved by at most
+        // one ulp of 1 - omega/2 where needed), so that the momentum a step adds,
+        // omega F/2 + (1 - omega/2) F, is exactly F; the Shan-Chen shift
+        // tau = 1/omega as hi + lo.
+        k.A = C(p.A);
+        k.h_e = C(1.0f - 0.5f * float(p.s_e));
+        k.h_eps = C(1.0f - 0.5f * float(p.s_eps));
+        k.h_q = C(1.0f - 0.5f * float(p.s_q));
         float om = float(1.0 / p.tau);
         float gp = float(1.0 - 0.5 * double(om));
         if (double(gp) != 1.0 - 0.5 * double(om)) om = float(2.0 * (1.0 - double(gp)));
@@ -81,7 +100,7 @@ lbm::Coef<C> make_coef(const lbm_params& p)
         const double t = 1.0 / double(om);
         k.tau = C(t);
         k.tau_lo = C(t - double(k.tau));
+        return k;
     }
-    return k;
 }
 #endif  // __CUDACC__ || LBM_HOST_ARITHMETIC
