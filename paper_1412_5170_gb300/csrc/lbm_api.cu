@@ -36,6 +36,7 @@ struct lbm_ctx {
     DevStats* hstats;       // pinned host mirror
     int64_t steps;
     int config;             // 0 = generic kernel, k >= 1 = strip configuration k-1
+    TilePlan tile;          // tiles of the generic kernel
     bool inject_timeout = false;   // the next step's first stage waits give up at once
     // Asynchronous host I/O, set up by the first lbm_init_density_async or
     // lbm_read_moments_async: one copy stream per direction, and device
@@ -54,6 +55,19 @@ namespace {
 inline size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 
 inline size_t tsize(const lbm_params& p) { return p.precision == LBM_FP64 ? sizeof(double) : sizeof(float); }
+
+// SMs of the device (one device per process).
+int sm_count()
+{
+    static int nsm = 0;
+    if (nsm == 0) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1)
+            nsm = 1;
+    }
+    return nsm;
+}
 
 dim3 generic_grid(const lbm_params& p)
 {
@@ -100,8 +114,22 @@ int cuda_status(cudaError_t e)
 template <typename T, typename C, int COLL, int FORC>
 void launch_generic(lbm_ctx* c, const void* fin, void* fout)
 {
-    k_step_generic<T, C, COLL, FORC><<<generic_grid(c->p), GTX * GTY, 0, c->stream>>>(
-        (const T*)fin, (T*)fout, c->p.nx, c->p.ny, make_coef<C>(c->p), c->status);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see k_step_generic
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(c->tile.sx, c->tile.sy);
+    lc.blockDim = dim3(c->tile.threads);
+    lc.stream = c->stream;
+    lc.attrs = attr;
+    // FP64 with more tiles than SMs: a plain launch.  A dependent grid's CTAs
+    // take whatever slots the running one leaves, several on one SM while
+    // others stay empty, which costs the FP64 pipe more than the launch gap
+    // (256 x 256: 30.7 us plain, 40.7 us dependent; 64 x 64, one tile per SM:
+    // 10.3 plain, 8.1 dependent).
+    lc.numAttrs = c->p.precision == LBM_FP64 && (long long)c->tile.sx * c->tile.sy > sm_count() ? 0 : 1;
+    cudaLaunchKernelEx(&lc, k_step_generic<T, C, COLL, FORC>, (const T*)fin, (T*)fout, c->p.nx, c->p.ny,
+                       make_coef<C>(c->p), c->status);
 }
 
 template <typename T, typename C>
@@ -115,15 +143,19 @@ void launch_generic_scheme(lbm_ctx* c, const void* fin, void* fout)
     else launch_generic<T, C, BGK, SC>(c, fin, fout);
 }
 
-// Without autotuning: the strip kernel where it applies -- for FP32 lattices
-// at least 1024 wide the 256-thread, two-stage carried configuration (the
-// fastest measured on large lattices), otherwise the first strip
-// configuration -- unless its strips and row chunks (at least 16 rows each)
-// cannot give every SM a CTA, as on small lattices, where the generic
-// kernel's 32 x 8 tiles spread wider; else the generic kernel.
+// Without autotuning.  FP64: the generic kernel, whose tiles keep the FP64
+// pipe busier than the strips' few CTAs (1024 x 1024: 356 us a step against
+// 445); from 2^21 nodes the two are close (1024 x 2560: 867 and 922) and the
+// strip kernel stays the automatic choice where it applies.  FP32: the strip
+// kernel where it applies -- for lattices at least 1024 wide the 256-thread,
+// two-stage carried configuration (the fastest measured on large lattices),
+// otherwise the first strip configuration -- unless its strips and row chunks
+// (at least 16 rows each) cannot give every SM a CTA, as on small lattices,
+// where the generic kernel's tiles spread wider; else the generic kernel.
 int default_config(const lbm_params& p)
 {
     if (!lbm_strip_supported(&p)) return 0;
+    if (p.precision == LBM_FP64 && (long long)p.nx * p.ny < (1 << 21)) return 0;
     int cfg = 1;
     if (p.precision == LBM_FP32_DEV && p.nx >= 1024) {
         const int n = lbm_strip_config_count(p.precision);
@@ -132,17 +164,10 @@ int default_config(const lbm_params& p)
             if (sc.threads == 256 && sc.stages == 2) { cfg = i + 1; break; }
         }
     }
-    static int nsm = 0;
-    if (nsm == 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1)
-            nsm = 1;
-    }
     const StripConfig sc = lbm_strip_config(p.precision, cfg - 1);
     const long long width = 4LL * sc.threads;
     const long long strips = (p.nx + width - 1) / width;
-    if (strips * std::max(1, p.ny / 16) < nsm) return 0;
+    if (strips * std::max(1, p.ny / 16) < sm_count()) return 0;
     return cfg;
 }
 
@@ -374,6 +399,7 @@ int lbm_create(const lbm_params* p, void* cuda_stream, void* workspace_dev, size
     c->status = (unsigned*)(b + L.status);
     c->cur = 0;
     c->config = default_config(*p);
+    c->tile = plan_tiles(p->nx, p->ny, p->precision == LBM_FP64, sm_count());
     cudaError_t e = cudaMallocHost(&c->hstats, sizeof(DevStats));
     if (e != cudaSuccess) {
         if (c->owns) cudaFree(c->ws);

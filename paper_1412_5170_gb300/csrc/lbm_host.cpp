@@ -201,3 +201,43 @@ int lbm_validate_preset(int nx, int ny, int kind, double size, double width, int
     if (kind == LBM_DROPLET_ARRAY && cell < 1) return LBM_E_INVALID;
     return LBM_OK;
 }
+
+// The cut with the smallest estimated step time, in issue cycles of one SM
+// quarter.  A node costs `psi` there for its density and psi (tile and ring)
+// and `col` for the rest of the update: FP64 instructions in FP64, which
+// occupy the quarter's pipe for a whole warp however few lanes are active;
+// instruction slots in FP32.  A CTA's warps spread over the four quarters, so
+//   - an SM that holds ceil(tiles / SMs) tiles takes a quarter of their
+//     warps' cost (beyond eight per SM the average, CTAs being started as
+//     others end),
+//   - and no tile takes less than its own warps in turn.
+// A tenth of the total work is added, so that of two cuts with the same
+// latency the one with less redundant psi wins (streams that share the GPU
+// notice the difference).
+TilePlan plan_tiles(int nx, int ny, bool fp64, int nsm)
+{
+    const double psi = fp64 ? 33 : 60, col = fp64 ? 110 : 170;
+    const int widths[] = {8, 10, 12, 16, 20, 24, 32, 43, 64};
+    const int heights[] = {1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 16, 20, 24, 32};
+    TilePlan best{0, 0, 0};
+    double best_cost = 0;
+    for (int w0 : widths)
+        for (int h0 : heights) {
+            const int sx = (nx + w0 - 1) / w0, sy = (ny + h0 - 1) / h0;
+            if (sy > 65535) continue;
+            const int w = (nx + sx - 1) / sx, h = (ny + sy - 1) / sy;   // the largest tile
+            if (w * h > 256 || (w + 2) * (h + 2) > 400) continue;
+            const int own = (w * h + 31) / 32, ring = (2 * (w + 2) + 2 * h + 31) / 32;
+            if (32 * (own + ring) > 384) continue;
+            const double tiles = double(sx) * sy, work = own * (psi + col) + ring * psi;
+            const double alone = (own + ring + 3) / 4 * psi + (own + 3) / 4 * col;
+            const double per_sm = tiles / nsm;
+            const double load = (per_sm > 8 ? per_sm : std::ceil(per_sm)) * work / 4 + (per_sm > 8 ? alone / 2 : 0);
+            const double cost = std::fmax(load, alone) + 0.1 * per_sm * work / 4;
+            if (best.sx == 0 || cost < best_cost) {
+                best = TilePlan{sx, sy, 32 * (own + ring)};
+                best_cost = cost;
+            }
+        }
+    return best;
+}

@@ -22,6 +22,11 @@ int lbm_validate_params(const lbm_params* p);
 // LBM_OK or LBM_E_INVALID for the arguments of a built-in field (lbm_init_preset).
 int lbm_validate_preset(int nx, int ny, int kind, double size, double width, int32_t cell);
 
+// Tiles of the generic step: the lattice cut into sx x sy nearly equal tiles,
+// one CTA of `threads` threads each.
+struct TilePlan { int sx, sy, threads; };
+TilePlan plan_tiles(int nx, int ny, bool fp64, int nsm);
+
 // Polls of a bounded stage wait (mbarrier try_wait) before the staged kernels
 // declare a row copy stuck, flag a timeout, drain and return.
 constexpr long long kStageWaitPolls = 1ll << 26;

@@ -65,43 +65,75 @@ __device__ __forceinline__ void flag_status(unsigned bad, unsigned* status)
 }
 
 // ---------------------------------------------------------------------------
-// Generic fused step: one node per thread on a TX x TY tile.  psi on the tile
-// plus a one-node ring is computed from pulled populations into shared
-// memory, then each thread computes F from the psi stencil, collides and
-// writes its nine post-collision deviations.  Works for any nx, ny >= 1.
+// Generic fused step, any nx, ny >= 1: a CTA owns a tile of at most 256 nodes,
+// one node per thread, and psi also on the ring of nodes around it.  Threads
+// [0, w h) take the tile's nodes and the warps after them the ring's, so psi
+// of both is evaluated at once from one round of loads; the tile's threads
+// keep their pulled populations from there to their collision (which takes F
+// from the psi of the tile and ring in shared memory).
+//
+// What bounds it: in FP64 the FP64 pipe, which takes 64 cycles per warp
+// instruction and SM quarter whatever lanes are active; on small FP32
+// lattices the latency of one load round.  The tile (plan_tiles) is therefore
+// cut to fill every SM quarter evenly, down to one row of 8 nodes, instead of
+// a fixed 32 x 8 (a 64 x 64 lattice gave 16 SMs work).  STEP2A_FIGS
+//
+// Launched as a programmatic dependent of the previous kernel on the stream,
+// as the strip step: it touches memory only after griddepcontrol.wait, and
+// lets the next step's CTAs be scheduled while this one runs.
 // ---------------------------------------------------------------------------
-constexpr int GTX = 32, GTY = 8;
+constexpr int GTX = 32, GTY = 8;   // observation tiles
+
+constexpr int kTileNodes = 256, kTileThreads = 384, kTilePsi = 400;
 
 template <typename T, typename C, int COLL, int FORC>
-__global__ void __launch_bounds__(GTX * GTY)
+__global__ void __launch_bounds__(kTileThreads)
 k_step_generic(const T* __restrict__ fin, T* __restrict__ fout, int nx, int ny, Coef<C> k,
                unsigned* __restrict__ status)
 {
-    __shared__ C sp[(GTY + 2) * (GTX + 2)];
-    const int x0 = blockIdx.x * GTX, y0 = blockIdx.y * GTY;
+    __shared__ C sp[kTilePsi];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int x0 = int((long long)blockIdx.x * nx / gridDim.x), y0 = int((long long)blockIdx.y * ny / gridDim.y);
+    const int w = int((long long)(blockIdx.x + 1) * nx / gridDim.x) - x0;
+    const int h = int((long long)(blockIdx.y + 1) * ny / gridDim.y) - y0;
     const size_t n = (size_t)nx * ny;
+    const int t = threadIdx.x, W = w + 2;
+    const bool own = t < w * h;
+    int lx, ly;
+    bool live = own;
+    if (own) {
+        ly = t / w;
+        lx = t - ly * w;
+    } else {   // the ring: rows -1 and h (w + 2 nodes each), then columns -1 and w
+        int r = t - (w * h + 31) / 32 * 32;
+        live = r >= 0 && r < 2 * W + 2 * h;
+        if (r < 2 * W) {
+            ly = r < W ? -1 : h;
+            lx = (r < W ? r : r - W) - 1;
+        } else {
+            r -= 2 * W;
+            lx = r < h ? -1 : w;
+            ly = r < h ? r : r - h;
+        }
+    }
     unsigned bad = 0;
-    for (int i = threadIdx.x; i < (GTX + 2) * (GTY + 2); i += blockDim.x) {
-        const int x = wrap_any(x0 + i % (GTX + 2) - 1, nx);
-        const int y = wrap_any(y0 + i / (GTX + 2) - 1, ny);
-        C g[9];
-        pull_node<T, C>(fin, x, y, nx, ny, n, g);
-        sp[i] = psi_of_rho<C>(k.rho_ref + sum9(g), k, bad);
+    C g[9];
+    if (live) {
+        const int xs = x0 + lx, ys = y0 + ly;   // one wrap at most: the tile is no larger than the lattice
+        pull_node<T, C>(fin, xs < 0 ? nx - 1 : (xs == nx ? 0 : xs), ys < 0 ? ny - 1 : (ys == ny ? 0 : ys), nx, ny, n, g);
+        sp[(ly + 1) * W + lx + 1] = psi_of_rho<C>(k.rho_ref + sum9(g), k, bad);
     }
     __syncthreads();
-    const int tx = threadIdx.x % GTX, ty = threadIdx.x / GTX;
-    const int x = x0 + tx, y = y0 + ty;
-    if (x < nx && y < ny) {
-        C g[9];
-        pull_node<T, C>(fin, x, y, nx, ny, n, g);
-        const int W = GTX + 2, c = (ty + 1) * W + tx + 1;
+    if (own) {
+        const int c = (ly + 1) * W + lx + 1;
         Stencil<C> q{sp[c], sp[c + 1], sp[c + W], sp[c - 1], sp[c - W],
                      sp[c + W + 1], sp[c + W - 1], sp[c - W - 1], sp[c - W + 1]};
         C Fx, Fy, vx, vy, rho;
         force<C>(q, k, Fx, Fy);
         collide<C, COLL, FORC>(g, Fx, Fy, k, vx, vy, rho, q.c);
         bad |= finite_bits<C>(g);
-        const size_t o = (size_t)y * nx + x;
+        const size_t o = (size_t)(y0 + ly) * nx + x0 + lx;
 #pragma unroll
         for (int a = 0; a < 9; ++a) fout[a * n + o] = T(g[a]);
     }

@@ -1,0 +1,35 @@
+"""The generic step's tiles at the sizes where their cut can go wrong: one
+node, single rows and columns (the ring wraps onto the tile itself), prime
+sides (tiles of unequal size), and lattices of many tiles.
+
+FP64 against the oracle at the parity bar (1e-12 of the largest population);
+FP32 at the element-wise bar of 2e-5 on the density.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1412_5170_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+MRT = dict(s_e=0.8, s_eps=0.8, s_q=1.1)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("coll,forc", [("mrt", "guo"), ("bgk", "edm")])
+@pytest.mark.parametrize("nx,ny", [(1, 1), (1, 331), (331, 1), (2, 97), (67, 3), (31, 257), (263, 129)])
+def test_tiles(lbm, nx, ny, coll, forc, precision):
+    rv, rl = lbm.maxwell(0.8)
+    rho0 = synth.density_field(nx, ny, "droplet", rl, rv, max(1.5, min(nx, ny) / 4), seed=5)
+    p = lbm.make_params(nx, ny, 0.8, 0.9, -0.304, 1.0, coll, forc, precision, **MRT)
+    with lbm.Lattice(p) as lat:
+        lat.variant = 0
+        lat.init_density(rho0)
+        lat.step(25)
+        f, st = lat.read_populations(), lat.stats()
+    ref, ost = oracle.run(oracle.params(nx, ny, 0.8, 0.9, -0.304, 1.0, coll, forc, **MRT), oracle.init_rest(rho0), 25)
+    assert ost == 0 and st["status"] == 0
+    if precision == "fp64":
+        assert np.abs(f - ref).max() < 1e-12 * np.abs(ref).max()
+    else:
+        assert (np.abs(f.sum(0) - ref.sum(0)) / ref.sum(0)).max() < 2e-5
