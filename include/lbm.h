@@ -260,11 +260,10 @@ int lbm_inject_stage_timeout(lbm_ctx *ctx);
 /* Kernel variant in use: 0 = generic tiled kernel (any nx), 1 = pipelined
  * strip kernel (nx % 4 == 0).  lbm_set_variant forces one (1 selects the
  * first strip configuration; LBM_E_UNSUPPORTED if the lattice does not
- * allow it); -1 restores the automatic choice: for FP32 lattices the strip
- * kernel where it applies (at least 1024 wide: its 256-thread, two-stage
- * configuration) and its strips and row chunks can give every SM a CTA,
- * else, and for FP64 lattices, the generic kernel.  lbm_autotune picks by
- * timing. */
+ * allow it); -1 restores the automatic choice: the strip kernel where it
+ * applies (for FP32 lattices at least 1024 wide its 256-thread, two-stage
+ * configuration; FP64 from 2^21 nodes) and its strips and row chunks can give
+ * every SM a CTA, else the generic kernel.  lbm_autotune picks by timing. */
 int lbm_get_variant(lbm_ctx *ctx, int *variant);
 int lbm_set_variant(lbm_ctx *ctx, int variant);
 
