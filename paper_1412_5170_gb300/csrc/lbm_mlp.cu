@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "lbm.h"
+#include "lbm_async.cuh"
 
 namespace {
 
@@ -125,9 +126,10 @@ __global__ void k_gather(const float* __restrict__ src, const int* __restrict__ 
 // twenty (standardise, a GEMM per layer and direction, loss, bias sums, Adam,
 // two copies), each 3-15 us of latency for a few thousand outputs.  Every sum
 // keeps its order (k ascending, one fused multiply-add a term, from zero), so
-// the parameters come out bit for bit as from the layered kernels above.
-// 2000 rows in minibatches of 64, two epochs and the final loss: 8.43 ms layer
-// by layer, 1.31 ms so; 256 predictions 57 and 34 us with their copies.
+// predictions and gradients come out bit for bit as from the layered kernels.
+// 2000 rows in minibatches of 64, two epochs and the final loss: 8.45 ms layer
+// by layer, 1.06 ms so (of a minibatch's 15 us k_net takes 9, k_net_grad 2,
+// the rest is the two launches); 256 predictions 57 and 34 us with copies.
 // ---------------------------------------------------------------------------
 constexpr int kMaxLayers = 17;   // 16 hidden layers and the output
 
@@ -138,7 +140,8 @@ struct NetShape {
     int S[kMaxLayers];           // shared-memory row stride of W: a multiple of 4 floats, odd in 16-byte units,
                                  // so that 128-bit reads of one column block by 8 lanes hit all 32 banks
     int sw[kMaxLayers];          // shared-memory offset of W (floats)
-    int wsum;                    // shared-memory floats of all W
+    int sb[kMaxLayers];          // the same for its biases
+    int wsum;                    // shared-memory floats of all W and biases: the image k_net copies
     int asum, amax;              // padded activation floats of a row, the widest layer's
 };
 struct NetBufs {
@@ -150,106 +153,191 @@ enum : int { NET_PREDICT = 0, NET_LOSS = 1, NET_GRAD = 2 };
 
 __host__ __device__ constexpr int pad4(int n) { return (n + 3) & ~3; }
 
-__device__ __forceinline__ void cp_async16(float* dst, const float* src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async4(float* dst, const float* src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
-}
 __device__ __forceinline__ void pdl_wait_and_release()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// All layers for 2 RPT rows a CTA: forward, and with NET_GRAD the deltas back
-// to the first layer.  The weights (166 KB for 5-128-128-128-64) are copied
-// into shared memory at once, the first layer's apart so that it can start,
-// with padded rows that serve both directions without bank conflicts: forward
-// a lane reads 4 k of its output's row, backward consecutive lanes read
-// consecutive inputs of one row.  A thread keeps RPT rows' sums of one
-// output.  Bound by the serial sums (128 dependent FMAs a layer) and the
-// weight copy (L2 to one SM, 1-2 us), so rows are spread over many CTAs.
-template <int RPT, int MODE>
-__global__ void __launch_bounds__(256)
-k_net(NetShape sh, const float* __restrict__ params, NetScale sc, const float* __restrict__ X,
-      const float* __restrict__ Y, const int* __restrict__ perm, int n, NetBufs buf, float* __restrict__ out,
-      float* __restrict__ row_loss)
+// acc[r] += sum_k a[r][k] w[k] in ascending k, one fused multiply-add a term;
+// the next 16 terms' reads are under way while these are added.
+template <int RPT>
+__device__ __forceinline__ void dot_rows(float (&acc)[RPT], const float* __restrict__ w, const float* __restrict__ a,
+                                         int P, int n)
 {
-    constexpr int R = 2 * RPT, NT = 256;
+    float4 wn[4], an[RPT][4];
+    auto fetch = [&](int k) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            wn[q] = *reinterpret_cast<const float4*>(w + k + 4 * q);
+#pragma unroll
+            for (int r = 0; r < RPT; ++r) an[r][q] = *reinterpret_cast<const float4*>(a + r * P + k + 4 * q);
+        }
+    };
+    int k = 0;
+    if (n >= 16) fetch(0);
+    for (; k + 16 <= n; k += 16) {
+        float4 wc[4], ac[RPT][4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            wc[q] = wn[q];
+#pragma unroll
+            for (int r = 0; r < RPT; ++r) ac[r][q] = an[r][q];
+        }
+        if (k + 32 <= n) fetch(k + 16);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int r = 0; r < RPT; ++r) {
+                acc[r] = fmaf(ac[r][q].x, wc[q].x, acc[r]);
+                acc[r] = fmaf(ac[r][q].y, wc[q].y, acc[r]);
+                acc[r] = fmaf(ac[r][q].z, wc[q].z, acc[r]);
+                acc[r] = fmaf(ac[r][q].w, wc[q].w, acc[r]);
+            }
+    }
+    for (; k < n; ++k)
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) acc[r] = fmaf(a[r * P + k], w[k], acc[r]);
+}
+// The same down a column of W: acc[r] += sum_o d[r][o] w[o S].
+template <int RPT>
+__device__ __forceinline__ void dot_cols(float (&acc)[RPT], const float* __restrict__ w, int S,
+                                         const float* __restrict__ d, int P, int n)
+{
+    float wn[8];
+    float4 dn[RPT][2];
+    auto fetch = [&](int o) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) wn[q] = w[(o + q) * S];
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) {
+            dn[r][0] = *reinterpret_cast<const float4*>(d + r * P + o);
+            dn[r][1] = *reinterpret_cast<const float4*>(d + r * P + o + 4);
+        }
+    };
+    int o = 0;
+    if (n >= 8) fetch(0);
+    for (; o + 8 <= n; o += 8) {
+        float wc[8];
+        float4 dc[RPT][2];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) wc[q] = wn[q];
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) {
+            dc[r][0] = dn[r][0];
+            dc[r][1] = dn[r][1];
+        }
+        if (o + 16 <= n) fetch(o + 8);
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+            for (int r = 0; r < RPT; ++r) {
+                acc[r] = fmaf(dc[r][q].x, wc[4 * q], acc[r]);
+                acc[r] = fmaf(dc[r][q].y, wc[4 * q + 1], acc[r]);
+                acc[r] = fmaf(dc[r][q].z, wc[4 * q + 2], acc[r]);
+                acc[r] = fmaf(dc[r][q].w, wc[4 * q + 3], acc[r]);
+            }
+    }
+    for (; o < n; ++o)
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) acc[r] = fmaf(d[r * P + o], w[o * S], acc[r]);
+}
+
+// All layers for H RPT rows a CTA: forward, and with NET_GRAD the deltas back
+// to the first layer.  Weights and biases (175 KB for 5-128-128-128-64) come
+// from `image`, which holds them as shared memory wants them: rows padded so
+// that both directions read without bank conflicts (forward a lane reads 4 k
+// of its output's row, backward consecutive lanes consecutive inputs of one
+// row), in a few bulk copies.  A thread keeps RPT rows' sums of one output.
+// Bound by latency: the serial sums (128 dependent FMAs a layer, 1 000 cycles
+// with their shared-memory reads) and the image's way from L2 to one SM; rows
+// are therefore spread over many CTAs.  (Copied out of the parameters row by
+// row -- cp.async of 16 bytes or a bulk copy a row -- issuing alone took
+// 5 000 to 9 000 cycles.)
+template <int H, int RPT, int MODE>
+__global__ void __launch_bounds__(256, 1)
+k_net(NetShape sh, const float* __restrict__ image, NetScale sc, const float* __restrict__ X,
+      const float* __restrict__ Y, const int* __restrict__ perm, int n, NetBufs buf, float* __restrict__ out,
+      float* __restrict__ row_loss, int* __restrict__ timeout)
+{
+    constexpr int R = H * RPT, NT = 256;
     extern __shared__ __align__(16) float sm[];
     float* const act = sm + sh.wsum;              // [layer][R][pad4(size)]
     float* const dl = act + R * sh.asum;          // two delta rows sets [2][R][amax]
+    float* const ty = dl + 2 * R * sh.amax;       // standardised targets [R][m]
+    uint64_t* const bar = reinterpret_cast<uint64_t*>(ty + pad4(R * sh.size[sh.L]));
     const int t = threadIdx.x, L = sh.L, r0 = blockIdx.x * R;
+    if (t == 0) {
+        lbm::mbar_init(bar, 1);
+        lbm::fence_mbar_init();
+    }
     pdl_wait_and_release();
-    for (int l = 0; l < L; ++l) {
-        const int in = sh.size[l], on = sh.size[l + 1], S = sh.S[l];
-        const float* W = params + sh.w[l];
-        float* d = sm + sh.sw[l];
-        if (((in | sh.w[l]) & 3) == 0) {
-            const int q = in >> 2;
-            for (int i = t; i < on * q; i += NT) {
-                const int o = i / q, c = (i - o * q) << 2;
-                cp_async16(d + o * S + c, W + o * in + c);
-            }
-        } else {
-            for (int i = t; i < on * in; i += NT) {
-                const int o = i / in;
-                cp_async4(d + o * S + (i - o * in), W + i);
-            }
-        }
-        if (l == 0) asm volatile("cp.async.commit_group;" ::: "memory");
+    if (t == 0) {
+        lbm::mbar_arrive_expect_tx(bar, 4u * sh.wsum);
+        for (int i = 0; i < sh.wsum; i += 4096) lbm::bulk_g2s(sm + i, image + i, 4u * min(4096, sh.wsum - i), bar);
     }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    {   // standardised inputs, (x - mean) / std per column
-        const int d = sh.size[0], P = pad4(d);
-        for (int i = t; i < R * d; i += NT) {
-            const int r = i / d, c = i - r * d;
-            float v = 0.f;
-            if (r0 + r < n) {
-                const int row = perm ? perm[r0 + r] : r0 + r;
-                v = (X[(size_t)row * d + c] - sc.xm[c]) / sc.xs[c];
-                if (MODE == NET_GRAD) buf.act[0][(size_t)(r0 + r) * d + c] = v;
-            }
-            act[r * P + c] = v;
+    // this thread's first input and target: every global read of the row block is under way at once
+    const int d0 = sh.size[0], m = sh.size[L];
+    const int xr = t / d0, xc = t - xr * d0, yr = t / m, yc = t - yr * m;
+    const bool hx = t < R * d0 && r0 + xr < n, hy = MODE != NET_PREDICT && t < R * m && r0 + yr < n;
+    const int xrow = hx ? (perm ? perm[r0 + xr] : r0 + xr) : 0, yrow = hy ? (perm ? perm[r0 + yr] : r0 + yr) : 0;
+    // (x - mean) / std per column
+    const int P0 = pad4(d0);
+    auto input = [&](int r, int c, float x, float mean, float sd) {
+        const float v = (x - mean) / sd;
+        if (MODE == NET_GRAD) buf.act[0][(size_t)(r0 + r) * d0 + c] = v;
+        act[r * P0 + c] = v;
+    };
+    {
+        float x = 0.f, xm = 0.f, xs = 1.f, y = 0.f, ym = 0.f, ys = 1.f;
+        if (hx) {
+            x = X[(size_t)xrow * d0 + xc];
+            xm = sc.xm[xc];
+            xs = sc.xs[xc];
+        }
+        if (hy) {
+            y = Y[(size_t)yrow * m + yc];
+            ym = sc.ym[yc];
+            ys = sc.ys[yc];
+        }
+        if (hx) input(xr, xc, x, xm, xs);
+        else if (t < R * d0) act[xr * P0 + xc] = 0.f;
+        if (hy) ty[t] = (y - ym) / ys;
+    }
+    for (int i = t + NT; i < R * d0; i += NT) {   // inputs and targets beyond one a thread
+        const int r = i / d0, c = i - r * d0;
+        if (r0 + r < n) input(r, c, X[(size_t)(perm ? perm[r0 + r] : r0 + r) * d0 + c], sc.xm[c], sc.xs[c]);
+        else act[r * P0 + c] = 0.f;
+    }
+    if (MODE != NET_PREDICT) {
+        for (int i = t + NT; i < R * m; i += NT) {
+            const int r = i / m, j = i - r * m;
+            if (r0 + r < n) ty[i] = (Y[(size_t)(perm ? perm[r0 + r] : r0 + r) * m + j] - sc.ym[j]) / sc.ys[j];
         }
     }
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    __syncthreads();
+    __syncthreads();   // the barrier is initialised, inputs and targets are in place
+    const bool ok = lbm::mbar_wait(bar, 0);
+    if (__syncthreads_or(!ok)) {   // the bounded wait gave up: flag it, wait once more for the copies, stop
+        if (t == 0) {
+            *timeout = 1;
+            lbm::mbar_wait(bar, 0);
+        }
+        __syncthreads();
+        return;
+    }
     float* ain = act;
     for (int l = 0; l < L; ++l) {
-        if (l == 1) {
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-            __syncthreads();
-        }
         const int in = sh.size[l], on = sh.size[l + 1], P = pad4(in), Q = pad4(on);
         float* aout = ain + R * P;
-        for (int i = t; i < 2 * on; i += NT) {
-            const int half = i >= on, o = i - half * on;
+        for (int i = t; i < H * on; i += NT) {
+            const int half = H > 1 && i >= on, o = i - half * on;
             const float* W = sm + sh.sw[l] + o * sh.S[l];
             const float* a = ain + half * RPT * P;
+            const float bias = sm[sh.sb[l] + o];
             float acc[RPT];
 #pragma unroll
             for (int r = 0; r < RPT; ++r) acc[r] = 0.f;
-            int k = 0;
-#pragma unroll 4
-            for (; k + 4 <= in; k += 4) {
-                const float4 w = *reinterpret_cast<const float4*>(W + k);
-#pragma unroll
-                for (int r = 0; r < RPT; ++r) {
-                    const float4 v = *reinterpret_cast<const float4*>(a + r * P + k);
-                    acc[r] = fmaf(v.x, w.x, acc[r]);
-                    acc[r] = fmaf(v.y, w.y, acc[r]);
-                    acc[r] = fmaf(v.z, w.z, acc[r]);
-                    acc[r] = fmaf(v.w, w.w, acc[r]);
-                }
-            }
-            for (; k < in; ++k)
-#pragma unroll
-                for (int r = 0; r < RPT; ++r) acc[r] = fmaf(a[r * P + k], W[k], acc[r]);
-            const float bias = params[sh.b[l] + o];
+            dot_rows<RPT>(acc, W, a, P, in);
 #pragma unroll
             for (int r = 0; r < RPT; ++r) {
                 const int row = half * RPT + r;
@@ -268,15 +356,13 @@ k_net(NetShape sh, const float* __restrict__ params, NetScale sc, const float* _
     }
     if (MODE == NET_PREDICT) return;
     // MSE in standardised units: d = out - t, delta = 2 d / (n m), and per row the sum of d^2
-    const int m = sh.size[L], Q = pad4(m);
+    const int Q = pad4(m);
     const float inv = 2.f / (float(n) * float(m));
     for (int i = t; i < R * m; i += NT) {
         const int r = i / m, j = i - r * m;
         float d = 0.f;
         if (r0 + r < n) {
-            const int row = perm ? perm[r0 + r] : r0 + r;
-            const float y = (Y[(size_t)row * m + j] - sc.ym[j]) / sc.ys[j];
-            d = ain[r * Q + j] - y;
+            d = ain[r * Q + j] - ty[i];
             if (MODE == NET_GRAD) buf.delta[L][(size_t)(r0 + r) * m + j] = inv * d;
         }
         if (MODE == NET_GRAD) dl[r * sh.amax + j] = inv * d;
@@ -297,30 +383,13 @@ k_net(NetShape sh, const float* __restrict__ params, NetScale sc, const float* _
         const int in = sh.size[l], on = sh.size[l + 1], P = pad4(in), S = sh.S[l];
         a -= R * P;
         const float* W = sm + sh.sw[l];
-        for (int i = t; i < 2 * in; i += NT) {
-            const int half = i >= in, c = i - half * in;
+        for (int i = t; i < H * in; i += NT) {
+            const int half = H > 1 && i >= in, c = i - half * in;
             const float* d = dcur + half * RPT * sh.amax;
             float acc[RPT];
 #pragma unroll
             for (int r = 0; r < RPT; ++r) acc[r] = 0.f;
-            int o = 0;
-#pragma unroll 4
-            for (; o + 4 <= on; o += 4) {
-                float w[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) w[q] = W[(o + q) * S + c];
-#pragma unroll
-                for (int r = 0; r < RPT; ++r) {
-                    const float4 v = *reinterpret_cast<const float4*>(d + r * sh.amax + o);
-                    acc[r] = fmaf(v.x, w[0], acc[r]);
-                    acc[r] = fmaf(v.y, w[1], acc[r]);
-                    acc[r] = fmaf(v.z, w[2], acc[r]);
-                    acc[r] = fmaf(v.w, w[3], acc[r]);
-                }
-            }
-            for (; o < on; ++o)
-#pragma unroll
-                for (int r = 0; r < RPT; ++r) acc[r] = fmaf(d[r * sh.amax + o], W[o * S + c], acc[r]);
+            dot_cols<RPT>(acc, W + c, S, d, sh.amax, on);
 #pragma unroll
             for (int r = 0; r < RPT; ++r) {
                 const int row = half * RPT + r;
@@ -343,8 +412,8 @@ k_net(NetShape sh, const float* __restrict__ params, NetScale sc, const float* _
 // them.
 template <bool ADAM>
 __global__ void __launch_bounds__(256)
-k_net_grad(NetShape sh, NetBufs buf, int n, float* __restrict__ params, float* __restrict__ grads,
-           float* __restrict__ m1, float* __restrict__ m2, Adam h)
+k_net_grad(NetShape sh, NetBufs buf, int n, float* __restrict__ params, float* __restrict__ image,
+           float* __restrict__ grads, float* __restrict__ m1, float* __restrict__ m2, Adam h)
 {
     __shared__ float sd[64][TS], sa[64][TS];
     int l = 0, tile = blockIdx.x, ti = 0;
@@ -358,13 +427,30 @@ k_net_grad(NetShape sh, NetBufs buf, int n, float* __restrict__ params, float* _
     const int o0 = (tile / ti) * TS, i0 = (tile % ti) * TS;
     const int t = threadIdx.x, tx = t % TS, ty = t / TS;
     const int o = o0 + ty, i = i0 + tx;
+    const bool wt = o < on && i < in, bias = o < on && i0 == 0 && tx == 0;
+    const int at = sh.w[l] + o * in + i, bt = sh.b[l] + o;
     pdl_wait_and_release();
+    // the parameters' Adam state is fetched under the sums
+    float p = 0.f, u = 0.f, v = 0.f;
+    if (ADAM && wt) {
+        p = params[at];
+        u = m1[at];
+        v = m2[at];
+    }
     float acc = 0.f, bsum = 0.f;
     for (int b0 = 0; b0 < n; b0 += 64) {
         const int nb = min(64, n - b0);
-        for (int q = ty; q < nb; q += 256 / TS) {
-            sd[q][tx] = o0 + tx < on ? buf.delta[l + 1][(size_t)(b0 + q) * on + o0 + tx] : 0.f;
-            sa[q][tx] = i < in ? buf.act[l][(size_t)(b0 + q) * in + i] : 0.f;
+        float rd[4], ra[4];   // all eight reads in flight together
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int q = ty + TS * j;
+            rd[j] = q < nb && o0 + tx < on ? buf.delta[l + 1][(size_t)(b0 + q) * on + o0 + tx] : 0.f;
+            ra[j] = q < nb && i < in ? buf.act[l][(size_t)(b0 + q) * in + i] : 0.f;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            sd[ty + TS * j][tx] = rd[j];
+            sa[ty + TS * j][tx] = ra[j];
         }
         __syncthreads();
         if (nb == 64) {
@@ -381,16 +467,38 @@ k_net_grad(NetShape sh, NetBufs buf, int n, float* __restrict__ params, float* _
         }
         __syncthreads();
     }
-    if (o >= on) return;
-    if (i < in) {
-        const int at = sh.w[l] + o * in + i;
-        if (ADAM) adam_update(params + at, acc, m1 + at, m2 + at, h);
-        else grads[at] = acc;
+    if (wt) {
+        if (ADAM) {
+            adam_update(&p, acc, &u, &v, h);
+            params[at] = p;
+            image[sh.sw[l] + o * sh.S[l] + i] = p;
+            m1[at] = u;
+            m2[at] = v;
+        } else {
+            grads[at] = acc;
+        }
     }
-    if (i0 == 0 && tx == 0) {
-        const int at = sh.b[l] + o;
-        if (ADAM) adam_update(params + at, bsum, m1 + at, m2 + at, h);
-        else grads[at] = bsum;
+    if (bias) {
+        if (ADAM) {
+            adam_update(params + bt, bsum, m1 + bt, m2 + bt, h);
+            image[sh.sb[l] + o] = params[bt];
+        } else {
+            grads[bt] = bsum;
+        }
+    }
+}
+
+// The image of the parameters (padding zero).
+__global__ void k_net_image(NetShape sh, const float* __restrict__ params, float* __restrict__ image)
+{
+    for (int l = 0; l < sh.L; ++l) {
+        const int in = sh.size[l], on = sh.size[l + 1], S = sh.S[l];
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < on * S; i += gridDim.x * blockDim.x) {
+            const int o = i / S, c = i - o * S;
+            image[sh.sw[l] + i] = c < in ? params[sh.w[l] + o * in + c] : 0.f;
+        }
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < pad4(on); i += gridDim.x * blockDim.x)
+            image[sh.sb[l] + i] = i < on ? params[sh.b[l] + i] : 0.f;
     }
 }
 
@@ -423,8 +531,10 @@ struct lbm_ws {
     float *tX = nullptr, *tY = nullptr;
     int *perm[2] = {nullptr, nullptr}, *hperm[2] = {nullptr, nullptr};   // device, pinned host
     cudaEvent_t perm_read[2] = {nullptr, nullptr};                       // the copy of hperm[k] is done
+    int* timeout = nullptr;          // pinned host flag a kernel sets when its weight copies did not land
     bool fused = false;              // the weights fit in shared memory: k_net and k_net_grad
     NetShape shape;
+    float* image = nullptr;          // fused: weights and biases in k_net's shared-memory layout, kept with params
 };
 
 namespace {
@@ -491,7 +601,10 @@ int ensure_train(lbm_ws* w, int n)
 }
 
 // Shared memory of k_net for R rows a CTA.
-size_t net_smem(const NetShape& s, int R) { return sizeof(float) * (s.wsum + (size_t)R * (s.asum + 2 * s.amax)); }
+size_t net_smem(const NetShape& s, int R)
+{
+    return sizeof(float) * (s.wsum + (size_t)R * (s.asum + 2 * s.amax) + pad4(R * s.size[s.L])) + sizeof(uint64_t);
+}
 
 // Shape of the fused kernels; false if the weights and the widest row block
 // (8 rows) exceed the shared memory of an SM.
@@ -513,6 +626,8 @@ bool make_shape(const lbm_ws* w, NetShape& s)
         if ((s.S[l] / 4) % 2 == 0) s.S[l] += 4;
         s.sw[l] = (int)wsum;
         wsum += (size_t)s.S[l] * w->sizes[l + 1];
+        s.sb[l] = (int)wsum;
+        wsum += pad4(w->sizes[l + 1]);
         if (wsum > 60000) return false;
     }
     s.wsum = (int)wsum;
@@ -521,11 +636,19 @@ bool make_shape(const lbm_ws* w, NetShape& s)
     return net_smem(s, 8) <= 227 * 1024;
 }
 
-template <int RPT, int MODE>
+// The image after params were set.
+int refresh_image(lbm_ws* w)
+{
+    if (!w->fused) return LBM_OK;
+    k_net_image<<<64, 256, 0, w->stream>>>(w->shape, w->params, w->image);
+    return ok(cudaGetLastError());
+}
+
+template <int H, int RPT, int MODE>
 int launch_net(lbm_ws* w, const float* X, const float* Y, const int* perm, int n, float* out, float* row_loss)
 {
-    const size_t smem = net_smem(w->shape, 2 * RPT);
-    auto kern = k_net<RPT, MODE>;
+    const size_t smem = net_smem(w->shape, H * RPT);
+    auto kern = k_net<H, RPT, MODE>;
     static const cudaError_t set = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     W_CUDA(set);
     NetBufs buf;
@@ -538,14 +661,14 @@ int launch_net(lbm_ws* w, const float* X, const float* Y, const int* perm, int n
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3((n + 2 * RPT - 1) / (2 * RPT));
+    lc.gridDim = dim3((n + H * RPT - 1) / (H * RPT));
     lc.blockDim = dim3(256);
     lc.dynamicSmemBytes = smem;
     lc.stream = w->stream;
     lc.attrs = attr;
     lc.numAttrs = 1;
-    W_CUDA(cudaLaunchKernelEx(&lc, kern, w->shape, (const float*)w->params, NetScale{w->xm, w->xs, w->ym, w->ys}, X, Y,
-                              perm, n, buf, out, row_loss));
+    W_CUDA(cudaLaunchKernelEx(&lc, kern, w->shape, (const float*)w->image, NetScale{w->xm, w->xs, w->ym, w->ys}, X, Y,
+                              perm, n, buf, out, row_loss, w->timeout));
     return LBM_OK;
 }
 
@@ -555,9 +678,9 @@ int launch_net(lbm_ws* w, const float* X, const float* Y, const int* perm, int n
 template <int MODE>
 int run_net(lbm_ws* w, const float* X, const float* Y, const int* perm, int n, float* out, float* row_loss)
 {
-    if (n <= 2 * 152) return launch_net<1, MODE>(w, X, Y, perm, n, out, row_loss);
-    if (n <= 4 * 152) return launch_net<2, MODE>(w, X, Y, perm, n, out, row_loss);
-    return launch_net<4, MODE>(w, X, Y, perm, n, out, row_loss);
+    if (n <= 2 * 152) return launch_net<1, 2, MODE>(w, X, Y, perm, n, out, row_loss);
+    if (n <= 4 * 152) return launch_net<1, 4, MODE>(w, X, Y, perm, n, out, row_loss);
+    return launch_net<2, 4, MODE>(w, X, Y, perm, n, out, row_loss);
 }
 
 template <bool ADAM>
@@ -571,6 +694,9 @@ int run_net_grad(lbm_ws* w, int n, const Adam& h)
         buf.delta[l] = w->deltas[l];
         if (l < w->shape.L) ntiles += ((w->sizes[l] + TS - 1) / TS) * ((w->sizes[l + 1] + TS - 1) / TS);
     }
+    // the same shared-memory split as k_net: changing it between the two costs an SM drain a launch
+    static const cudaError_t set = cudaFuncSetAttribute(k_net_grad<ADAM>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    W_CUDA(set);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -580,7 +706,7 @@ int run_net_grad(lbm_ws* w, int n, const Adam& h)
     lc.stream = w->stream;
     lc.attrs = attr;
     lc.numAttrs = 1;
-    W_CUDA(cudaLaunchKernelEx(&lc, k_net_grad<ADAM>, w->shape, buf, n, w->params, w->grads, w->m1, w->m2, h));
+    W_CUDA(cudaLaunchKernelEx(&lc, k_net_grad<ADAM>, w->shape, buf, n, w->params, w->image, w->grads, w->m1, w->m2, h));
     return LBM_OK;
 }
 
@@ -626,6 +752,14 @@ int backward(lbm_ws* w, int n)
     return ok(cudaGetLastError());
 }
 
+// LBM_E_TIMEOUT (once) if a kernel before the last synchronisation gave up waiting.
+int timed_out(lbm_ws* w)
+{
+    if (!*w->timeout) return LBM_OK;
+    *w->timeout = 0;
+    return LBM_E_TIMEOUT;
+}
+
 // Loss over n rows X, Y on the device (mean squared error in standardised
 // units), and with grad its gradient into w->grads.
 int loss_of(lbm_ws* w, const float* X, const float* Y, int n, bool grad, float* loss)
@@ -644,6 +778,7 @@ int loss_of(lbm_ws* w, const float* X, const float* Y, int n, bool grad, float* 
     std::vector<float> rl(n);
     W_CUDA(cudaMemcpyAsync(rl.data(), w->rowloss, sizeof(float) * n, cudaMemcpyDeviceToHost, w->stream));
     W_CUDA(cudaStreamSynchronize(w->stream));
+    if ((s = timed_out(w)) != LBM_OK) return s;
     double tot = 0;
     for (float v : rl) tot += v;
     if (loss) *loss = float(tot / (double(n) * w->sizes.back()));
@@ -686,7 +821,10 @@ int lbm_ws_create(const lbm_ws_cfg* cfg, lbm_ws** out)
     std::vector<float> one_in(cfg->n_in, 1.f), zero_in(cfg->n_in, 0.f), one_out(cfg->n_out, 1.f),
         zero_out(cfg->n_out, 0.f);
     cudaError_t e = cudaStreamCreateWithFlags(&w->stream, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaMallocHost(&w->timeout, sizeof(int));
+    if (e == cudaSuccess) *w->timeout = 0;
     if (e == cudaSuccess) e = cudaMalloc(&w->params, sizeof(float) * p);
+    if (e == cudaSuccess && w->fused) e = cudaMalloc(&w->image, sizeof(float) * w->shape.wsum);
     if (e == cudaSuccess) e = cudaMalloc(&w->grads, sizeof(float) * p);
     if (e == cudaSuccess) e = cudaMalloc(&w->m1, sizeof(float) * p);
     if (e == cudaSuccess) e = cudaMalloc(&w->m2, sizeof(float) * p);
@@ -694,13 +832,15 @@ int lbm_ws_create(const lbm_ws_cfg* cfg, lbm_ws** out)
     if (e == cudaSuccess) e = cudaMalloc(&w->xs, sizeof(float) * cfg->n_in);
     if (e == cudaSuccess) e = cudaMalloc(&w->ym, sizeof(float) * cfg->n_out);
     if (e == cudaSuccess) e = cudaMalloc(&w->ys, sizeof(float) * cfg->n_out);
-    if (e == cudaSuccess) e = cudaMemcpy(w->params, h.data(), sizeof(float) * p, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(w->m1, 0, sizeof(float) * p);
-    if (e == cudaSuccess) e = cudaMemset(w->m2, 0, sizeof(float) * p);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(w->params, h.data(), sizeof(float) * p, cudaMemcpyHostToDevice, w->stream);
+    if (e == cudaSuccess && refresh_image(w) != LBM_OK) e = cudaErrorUnknown;
+    if (e == cudaSuccess) e = cudaMemsetAsync(w->m1, 0, sizeof(float) * p, w->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w->m2, 0, sizeof(float) * p, w->stream);
     if (e == cudaSuccess) e = cudaMemcpy(w->xm, zero_in.data(), sizeof(float) * cfg->n_in, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(w->xs, one_in.data(), sizeof(float) * cfg->n_in, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(w->ym, zero_out.data(), sizeof(float) * cfg->n_out, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(w->ys, one_out.data(), sizeof(float) * cfg->n_out, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(w->stream);
     if (e != cudaSuccess) {
         lbm_ws_destroy(w);
         return ok(e);
@@ -713,10 +853,12 @@ void lbm_ws_destroy(lbm_ws* w)
 {
     if (!w) return;
     if (w->stream) cudaStreamSynchronize(w->stream);
-    for (float* p : {w->params, w->grads, w->m1, w->m2, w->xm, w->xs, w->ym, w->ys, w->rowloss, w->X, w->Y, w->tX, w->tY})
+    for (float* p : {w->params, w->grads, w->m1, w->m2, w->xm, w->xs, w->ym, w->ys, w->rowloss, w->X, w->Y, w->tX, w->tY,
+                     w->image})
         cudaFree(p);
     for (float* p : w->acts) cudaFree(p);
     for (float* p : w->deltas) cudaFree(p);
+    if (w->timeout) cudaFreeHost(w->timeout);
     for (int k = 0; k < 2; ++k) {
         cudaFree(w->perm[k]);
         if (w->hperm[k]) cudaFreeHost(w->hperm[k]);
@@ -762,6 +904,8 @@ int lbm_ws_set_params(lbm_ws* w, const float* host)
     W_CUDA(cudaMemsetAsync(w->m1, 0, sizeof(float) * w->np, w->stream));
     W_CUDA(cudaMemsetAsync(w->m2, 0, sizeof(float) * w->np, w->stream));
     W_CUDA(cudaMemcpyAsync(w->params, host, sizeof(float) * w->np, cudaMemcpyHostToDevice, w->stream));
+    const int s = refresh_image(w);
+    if (s != LBM_OK) return s;
     W_CUDA(cudaStreamSynchronize(w->stream));
     w->t = 0;
     return LBM_OK;
@@ -828,6 +972,7 @@ int lbm_ws_train(lbm_ws* w, const float* X_host, const float* Y_host, int n, int
     }
     const int e = ok(cudaStreamSynchronize(w->stream));
     if (s == LBM_OK) s = e;
+    if (s == LBM_OK) s = timed_out(w);
     if (s == LBM_OK && final_loss)   // loss over the whole training set with the final parameters
         s = loss_of(w, w->tX, w->tY, n, false, final_loss);
     return s;
@@ -850,7 +995,7 @@ int lbm_ws_predict(lbm_ws* w, const float* X_host, int n, float* Y_host)
     }
     W_CUDA(cudaMemcpyAsync(Y_host, outp, sizeof(float) * n * m, cudaMemcpyDeviceToHost, w->stream));
     W_CUDA(cudaStreamSynchronize(w->stream));
-    return LBM_OK;
+    return timed_out(w);
 }
 
 }  // extern "C"
