@@ -287,8 +287,8 @@ int lbm_autotune(lbm_ctx *ctx, int trial_steps, int *config, double *ms_per_step
  * Many independent periodic lattices with their own size, T/Tc, tau, A, K and
  * initial field (the paper's tau, T/Tc and EOS-scale sweeps, Secs. 4.2-4.4)
  * advanced together: one kernel launch per time step covers every running
- * instance through a table of (instance, column strip, row chunk) work
- * items, each check interval is one CUDA graph, and convergence or failure is
+ * instance through a table of (instance, column strip, row chunk) work items
+ * or of tiles, each check interval is one CUDA graph, and convergence or failure is
  * decided per instance on the device.  Populations are FP32 deviations
  * (precision must be LBM_FP32_DEV; rho_ref = the instance's Maxwell vapour
  * density); every nx must be a multiple of 4.  All batch calls are
@@ -421,10 +421,14 @@ int lbm_batch_profiles(lbm_batch *b, int nb, const lbm_profile_geom *geom_host, 
  *   columns 128: one warp walks a strip; stages 3 or 4 (carry 0), 2 or 3 (carry 1).
  *   columns 256: a 64-thread CTA walks a strip; stages 3, carry 1 only.
  *   columns 512: a 128-thread CTA walks a strip; stages 2 or 3, carry 1 only.
- * Other combinations return LBM_E_INVALID.  lbm_batch_autotune times the
- * seven (columns, stages, carry) candidates x rows 32, 64, 128, 256 for trial_steps
- * steps each without advancing the state and keeps the fastest; any output
- * pointer may be NULL. */
+ * Other combinations return LBM_E_INVALID.  Small batches (up to 2^23 running
+ * nodes) and narrow lattices step on tiles of at most 256 nodes instead,
+ * unless lbm_batch_set_tuning asked for a walk.  lbm_batch_autotune times the
+ * seven (columns, stages, carry) candidates x rows 32, 64, 128, 256 for
+ * trial_steps steps each without advancing the state, and the tiles where
+ * they apply, and keeps the fastest (columns .. carry then name the fastest
+ * walk, ms_per_step the time of what is kept); any output pointer may be
+ * NULL. */
 int lbm_batch_set_tuning(lbm_batch *b, int columns, int stages, int rows_per_item, int carry);
 int lbm_batch_autotune(lbm_batch *b, int trial_steps, int *columns, int *stages, int *rows_per_item, int *carry,
                        double *ms_per_step);

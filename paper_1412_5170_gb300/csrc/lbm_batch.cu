@@ -42,6 +42,8 @@ struct BPart {
 // deviation drho (rho = rho_ref + drho).
 struct __align__(16) Snap { float vx, vy, drho, pad; };
 
+constexpr long long kTileStepNodes = 1 << 23;   // see build_tiles
+
 constexpr int kBatchWarps = 1;   // warps (independent 128-column walkers) per CTA
 
 // Dynamic shared memory of one batched-step CTA: per warp its stage ring and
@@ -98,6 +100,36 @@ k_step_batch(const float* __restrict__ fin, float* __restrict__ fout, const BIns
             atomicExch(&queue[1], 0);
         }
     }
+}
+
+// The tiled step: one CTA per tile of the table, the generic kernel's update
+// (step_tile).  For batches too small or too narrow to fill the walks: a slab
+// of 8 columns leaves a 128-column walker 30 of its 32 lanes idle, and a walk
+// of a few rows is a chain of queue, copy and barrier latencies.  Here a step
+// is one round of loads, and consecutive steps are dependent launches whose
+// tile record and constants (written only between runs, on a synchronised
+// stream) are fetched before the wait.  Per step, walk and tiles: 24 slabs of
+// 8 x 128 20.6 and 2.5 us, one 64 x 64 lattice 19.5 and 2.0, 16 instances of
+// the sweep (2.0 M nodes) 58 and 40.
+template <int COLL, int FORC>
+__global__ void __launch_bounds__(kTileThreads)
+k_step_batch_tiles(const float* __restrict__ fin, float* __restrict__ fout, const BInst* __restrict__ inst,
+                   const BStepTile* __restrict__ tiles, const int* __restrict__ state, unsigned* __restrict__ inst_status)
+{
+    __shared__ float sp[kTilePsi];
+    __shared__ Coef<float> sk;
+    const BStepTile tl = tiles[blockIdx.x];
+    constexpr int nwords = sizeof(Coef<float>) / sizeof(float);
+    static_assert(nwords <= 32, "one warp stages the constants");
+    if (threadIdx.x < nwords)
+        reinterpret_cast<float*>(&sk)[threadIdx.x] = reinterpret_cast<const float*>(&inst[tl.inst].k)[threadIdx.x];
+    __syncthreads();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (state[tl.inst] != B_RUNNING) return;   // uniform over the CTA
+    unsigned bad = 0;
+    step_tile<float, float, COLL, FORC>(fin + tl.off, fout + tl.off, tl.nx, tl.ny, tl.x0, tl.y0, tl.w, tl.h, sk, sp, bad);
+    flag_status(bad, &inst_status[tl.inst]);
 }
 
 template <int NS>
@@ -535,6 +567,10 @@ struct lbm_batch {
     int nitems = 0;
     int items_cap = 0;
     int items_for = 0;           // running instances when the work items were last built
+    BStepTile* stiles = nullptr; // tiles of the tiled step
+    int nstiles = 0, stiles_cap = 0, stile_threads = 0;
+    bool use_tiles = false;      // the tiled step instead of the walks
+    bool allow_tiles = true;     // false once a walk was asked for (lbm_batch_set_tuning) or timed faster
     int* state = nullptr;        // device
     int* fail = nullptr;         // device
     unsigned* status = nullptr;  // device, per instance
@@ -580,6 +616,66 @@ void drop_graphs(lbm_batch* b)
         if (g) { cudaGraphExecDestroy(g); g = nullptr; }
 }
 
+int batch_sms()
+{
+    static int nsm = 0;
+    if (nsm == 0) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1) nsm = 1;
+    }
+    return nsm;
+}
+
+// Tiles of the running instances for the tiled step, and whether it is used:
+// up to 2^23 nodes (64 instances of the sweep, 7.5 M nodes: 146 us a step
+// against the walk's 178; 256 instances, 25 M nodes, 484 against 462), and
+// for narrow lattices at any size (where whole strips would hold twice the
+// nodes; 200 slabs of 8 x 128: 5.9 us against 72.7).
+int build_tiles(lbm_batch* b, const int* host_state)
+{
+    const int nsm = batch_sms();
+    long long nodes = 0, padded = 0;   // nodes, and nodes of whole 128-column strips
+    for (int i = 0; i < b->n; ++i) {
+        if (host_state && host_state[i] != B_RUNNING) continue;
+        const BInst& I = b->hinst[i];
+        nodes += (long long)I.nx * I.ny;
+        padded += (long long)((I.nx + 127) / 128 * 128) * I.ny;
+    }
+    b->use_tiles = b->allow_tiles && (nodes <= kTileStepNodes || padded >= 2 * nodes);
+    b->nstiles = 0;
+    if (!b->use_tiles || nodes == 0) return LBM_OK;
+    // two tiles per SM where the batch is that small, 256 nodes at most (smaller ones cost more ring:
+    // 146, 163 and 213 us a step at 256, 128 and 64 nodes on 7.5 M nodes)
+    const int want = (int)std::min<long long>(256, std::max<long long>(32, nodes / (2 * nsm)));
+    std::vector<BStepTile> t;
+    b->stile_threads = 0;
+    for (int i = 0; i < b->n; ++i) {
+        if (host_state && host_state[i] != B_RUNNING) continue;
+        const BInst& I = b->hinst[i];
+        const int sx = (I.nx + 31) / 32, w = (I.nx + sx - 1) / sx;
+        const int h0 = std::min(32, std::max(1, want / w)), sy = (I.ny + h0 - 1) / h0, h = (I.ny + sy - 1) / sy;
+        b->stile_threads = std::max(b->stile_threads, 32 * ((w * h + 31) / 32 + (2 * (w + 2) + 2 * h + 31) / 32));
+        for (int ty = 0; ty < sy; ++ty)
+            for (int tx = 0; tx < sx; ++tx) {
+                const int x0 = int((long long)tx * I.nx / sx), x1 = int((long long)(tx + 1) * I.nx / sx);
+                const int y0 = int((long long)ty * I.ny / sy), y1 = int((long long)(ty + 1) * I.ny / sy);
+                t.push_back(BStepTile{I.off, i, I.nx, I.ny, x0, y0, x1 - x0, y1 - y0, 0});
+            }
+    }
+    if ((int)t.size() > b->stiles_cap) {
+        if (b->stiles) cudaFree(b->stiles);
+        b->stiles = nullptr;
+        b->stiles_cap = 0;
+        B_CUDA(cudaMalloc(&b->stiles, sizeof(BStepTile) * t.size()));
+        b->stiles_cap = (int)t.size();
+    }
+    B_CUDA(cudaMemcpyAsync(b->stiles, t.data(), sizeof(BStepTile) * t.size(), cudaMemcpyHostToDevice, b->stream));
+    B_CUDA(cudaStreamSynchronize(b->stream));
+    b->nstiles = (int)t.size();
+    return LBM_OK;
+}
+
 // Work items of the running instances: strips of b->cols columns cut into
 // row chunks of about b->rows rows.  When the running instances hold too few strip rows
 // to give every SM about sixteen items at that length (small batches, and
@@ -588,12 +684,7 @@ void drop_graphs(lbm_batch* b)
 // batched-step SM holds) and its latency (one row walk) shortens.
 int build_items(lbm_batch* b, const int* host_state)
 {
-    static int nsm = 0;
-    if (nsm == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1) nsm = 1;
-    }
+    const int nsm = batch_sms();
     long long strip_rows = 0;
     for (int i = 0; i < b->n; ++i) {
         if (host_state && host_state[i] != B_RUNNING) continue;
@@ -631,7 +722,37 @@ int build_items(lbm_batch* b, const int* host_state)
         B_CUDA(cudaMemcpyAsync(b->items, it.data(), sizeof(BItem) * b->nitems, cudaMemcpyHostToDevice, b->stream));
     B_CUDA(cudaStreamSynchronize(b->stream));
     drop_graphs(b);
-    return LBM_OK;
+    return build_tiles(b, host_state);
+}
+
+template <int COLL, int FORC>
+int launch_tiles(lbm_batch* b, const float* fin, float* fout)
+{
+    cudaFuncAttributes fa;   // loads the kernel before any graph capture
+    static const cudaError_t loaded = cudaFuncGetAttributes(&fa, k_step_batch_tiles<COLL, FORC>);
+    if (loaded != cudaSuccess) return LBM_E_CUDA;
+    if (b->nstiles == 0) return LBM_OK;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see k_step_batch_tiles
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(b->nstiles);
+    lc.blockDim = dim3(b->stile_threads);
+    lc.stream = b->stream;
+    lc.attrs = attr;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, k_step_batch_tiles<COLL, FORC>, fin, fout, (const BInst*)b->dinst,
+                              (const BStepTile*)b->stiles, (const int*)b->state, b->status) == cudaSuccess
+               ? LBM_OK : LBM_E_CUDA;
+}
+
+int launch_batch_tiles(lbm_batch* b, const float* fin, float* fout)
+{
+    if (b->collision == LBM_MRT) return launch_tiles<MRT, GUO>(b, fin, fout);
+    if (b->forcing == LBM_GUO) return launch_tiles<BGK, GUO>(b, fin, fout);
+    if (b->forcing == LBM_EDM) return launch_tiles<BGK, EDM>(b, fin, fout);
+    if (b->forcing == LBM_LI) return launch_tiles<BGK, LI>(b, fin, fout);
+    return launch_tiles<BGK, SC>(b, fin, fout);
 }
 
 template <int COLL, int FORC, int NS, bool CARRY>
@@ -686,7 +807,7 @@ int step_once(lbm_batch* b)
 {
     const float* fin = b->f[b->cur];
     float* fout = b->f[b->cur ^ 1];
-    const int s = launch_batch_tuned(b, fin, fout);
+    const int s = b->use_tiles ? launch_batch_tiles(b, fin, fout) : launch_batch_tuned(b, fin, fout);
     if (s != LBM_OK) return s;
     b->cur ^= 1;
     return LBM_OK;
@@ -851,6 +972,10 @@ int lbm_batch_create(const lbm_batch_params* bp, const lbm_instance* inst, int n
     if (s == LBM_OK) s = launch_batch_scheme<2, true>(b, b->f[0], b->f[1]);
     if (s == LBM_OK) s = launch_batch_scheme<3, true>(b, b->f[0], b->f[1]);
     b->nitems = saved;
+    const int saved_tiles = b->nstiles;
+    b->nstiles = 0;
+    if (s == LBM_OK) s = launch_batch_tiles(b, b->f[0], b->f[1]);
+    b->nstiles = saved_tiles;
     if (s != LBM_OK) { lbm_batch_destroy(b); return s; }
     std::fill(b->h_state, b->h_state + b->n, (int)B_RUNNING);
     *out = b;
@@ -870,6 +995,7 @@ void lbm_batch_destroy(lbm_batch* b)
     cudaFree(b->parts);
     cudaFree(b->tiles);
     cudaFree(b->items);
+    cudaFree(b->stiles);
     cudaFree(b->state);
     cudaFree(b->fail);
     cudaFree(b->status);
@@ -1091,6 +1217,7 @@ int lbm_batch_set_tuning(lbm_batch* b, int columns, int stages, int rows_per_ite
     b->ns = stages;
     b->carry = carry ? 1 : 0;
     b->rows = rows_per_item;
+    b->allow_tiles = false;
     return build_items(b, b->h_state);
 }
 
@@ -1132,14 +1259,32 @@ int lbm_batch_autotune(lbm_batch* b, int trial_steps, int* columns, int* stages,
             ms /= trial_steps;
             if (ms < best) { best = ms; bcols = b->cols; bns = b->ns; brows = b->rows; bcarry = b->carry; }
         }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
     b->cur = cur0;
     b->cols = bcols;
     b->ns = bns;
     b->rows = brows;
     b->carry = bcarry;
-    const int s = build_items(b, b->h_state);
+    // the tiled step, where it is the batch's automatic choice, against the best walk
+    b->allow_tiles = true;
+    int s = build_items(b, b->h_state);
+    if (status == LBM_OK && s == LBM_OK && b->use_tiles) {
+        const float* fin = b->f[cur0];
+        float* fout = b->f[cur0 ^ 1];
+        status = launch_batch_tiles(b, fin, fout);
+        cudaEventRecord(e0, b->stream);
+        for (int i = 0; i < trial_steps && status == LBM_OK; ++i) status = launch_batch_tiles(b, fin, fout);
+        cudaEventRecord(e1, b->stream);
+        if (status == LBM_OK) status = cuda_ok(cudaEventSynchronize(e1));
+        float ms = 0;
+        if (status == LBM_OK && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess && ms / trial_steps < best) {
+            best = ms / trial_steps;
+        } else {
+            b->allow_tiles = false;
+            s = build_items(b, b->h_state);
+        }
+    }
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
     if (status != LBM_OK) return status;
     if (s != LBM_OK) return s;
     if (columns) *columns = bcols;

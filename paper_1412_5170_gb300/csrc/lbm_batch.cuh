@@ -25,6 +25,9 @@ struct BInst {
 // instance inst; down: walk the chunk's rows downwards.
 struct BItem { int inst, x0, y0, y1, down, pad[3]; };
 
+// One tile of the tiled step: what a CTA needs to start its loads.
+struct BStepTile { long long off; int inst, nx, ny, x0, y0, w, h, pad; };
+
 enum : int { B_RUNNING = 0, B_CONVERGED = 1, B_FAILED = 2 };
 
 // Arguments of one batched-step launch.  queue: the work-item counter and

@@ -90,17 +90,12 @@ constexpr int GTX = 32, GTY = 8;   // observation tiles
 
 constexpr int kTileNodes = 256, kTileThreads = 384, kTilePsi = 400;
 
+// One tile [x0, x0 + w) x [y0, y0 + h) of an nx x ny lattice: every thread of
+// the CTA calls it, after its griddepcontrol.wait.
 template <typename T, typename C, int COLL, int FORC>
-__global__ void __launch_bounds__(kTileThreads)
-k_step_generic(const T* __restrict__ fin, T* __restrict__ fout, int nx, int ny, Coef<C> k,
-               unsigned* __restrict__ status)
+__device__ __forceinline__ void step_tile(const T* __restrict__ fin, T* __restrict__ fout, int nx, int ny, int x0, int y0,
+                                          int w, int h, const Coef<C>& k, C* __restrict__ sp, unsigned& bad)
 {
-    __shared__ C sp[kTilePsi];
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int x0 = int((long long)blockIdx.x * nx / gridDim.x), y0 = int((long long)blockIdx.y * ny / gridDim.y);
-    const int w = int((long long)(blockIdx.x + 1) * nx / gridDim.x) - x0;
-    const int h = int((long long)(blockIdx.y + 1) * ny / gridDim.y) - y0;
     const size_t n = (size_t)nx * ny;
     const int t = threadIdx.x, W = w + 2;
     const bool own = t < w * h;
@@ -121,7 +116,6 @@ k_step_generic(const T* __restrict__ fin, T* __restrict__ fout, int nx, int ny, 
             ly = r < h ? r : r - h;
         }
     }
-    unsigned bad = 0;
     C g[9];
     if (live) {
         const int xs = x0 + lx, ys = y0 + ly;   // one wrap at most: the tile is no larger than the lattice
@@ -141,6 +135,21 @@ k_step_generic(const T* __restrict__ fin, T* __restrict__ fout, int nx, int ny, 
 #pragma unroll
         for (int a = 0; a < 9; ++a) fout[a * n + o] = T(g[a]);
     }
+}
+
+template <typename T, typename C, int COLL, int FORC>
+__global__ void __launch_bounds__(kTileThreads)
+k_step_generic(const T* __restrict__ fin, T* __restrict__ fout, int nx, int ny, Coef<C> k,
+               unsigned* __restrict__ status)
+{
+    __shared__ C sp[kTilePsi];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int x0 = int((long long)blockIdx.x * nx / gridDim.x), y0 = int((long long)blockIdx.y * ny / gridDim.y);
+    const int w = int((long long)(blockIdx.x + 1) * nx / gridDim.x) - x0;
+    const int h = int((long long)(blockIdx.y + 1) * ny / gridDim.y) - y0;
+    unsigned bad = 0;
+    step_tile<T, C, COLL, FORC>(fin, fout, nx, ny, x0, y0, w, h, k, sp, bad);
     flag_status(bad, status);
 }
 
