@@ -137,17 +137,46 @@ constexpr size_t batch_smem() { return batch_coef_off<NS>() + kBatchWarps * size
 
 enum : int { BO_RHO = 1, BO_SNAP = 2, BO_ALL = 4 };
 
+// Sum of floats held as an unevaluated pair (s, e): Knuth's TwoSum keeps each
+// addition's rounding in e, so the pair is good to about 2^-45 without the
+// FP64 pipe.
+struct FPair { float s, e; };
+__device__ __forceinline__ FPair pair_add(FPair a, FPair b)
+{
+    const float t = a.s + b.s, bp = t - a.s;
+    return FPair{t, (a.e + b.e) + ((a.s - (t - bp)) + (b.s - bp))};
+}
+// Its value in FP64 (an infinite or NaN sum leaves no rounding to add).
+__device__ __forceinline__ double pair_value(FPair p) { return isfinite(p.e) ? double(p.s) + double(p.e) : double(p.s); }
+__device__ __forceinline__ FPair warp_pair_sum(float v)
+{
+    FPair p{v, 0.f};
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        p = pair_add(p, FPair{__shfl_xor_sync(0xffffffffu, p.s, o), __shfl_xor_sync(0xffffffffu, p.e, o)});
+    return p;
+}
+
 // Observables per 32 x 8 tile of every running instance (every instance with
 // BO_ALL): rho and v = u + F/(2 rho); with BO_SNAP the changes against the
 // snapshot (vx, vy, rho) of the previous check, which is then replaced; with
 // BO_RHO the FP64 density field.
-__global__ void __launch_bounds__(GTX * GTY)
+//
+// Eight warps take the tile's rows and three the ring of nodes around it, so
+// that every node is pulled and its psi evaluated once, from one round of
+// loads.  All per-node and per-warp work is FP32: maxima are exact in any
+// precision, the sums of drho are float pairs, and one thread per tile turns
+// seven numbers into FP64.  (With FP64 shuffle sums and the pull repeated
+// after the psi pass lbm_batch_observe took 1.57 ms on the 25 M nodes of 256
+// sweep instances; now 0.71, of which the populations' way from HBM is 0.13.)
+constexpr int kObsThreads = 32 * (GTY + 3);
+__global__ void __launch_bounds__(kObsThreads)
 k_observe_batch(const float* __restrict__ f, const BInst* __restrict__ inst, const BTile* __restrict__ tiles,
                 const int* __restrict__ state, Snap* __restrict__ snap, double* __restrict__ rho_out,
                 BPart* __restrict__ parts, BObs* __restrict__ obs, int mode)
 {
     __shared__ float sp[(GTY + 2) * (GTX + 2)];
-    __shared__ double red[8][GTX * GTY / 32];
+    __shared__ float red[11][GTY];
     __shared__ unsigned sbad;
     const BTile tl = tiles[blockIdx.x];
     if (!(mode & BO_ALL) && state[tl.inst] != B_RUNNING) return;   // uniform over the block
@@ -156,40 +185,55 @@ k_observe_batch(const float* __restrict__ f, const BInst* __restrict__ inst, con
     const Coef<float> k = I->k;
     const float* fi = f + I->off;
     const size_t n = (size_t)nx * ny;
-    const int x0 = tl.tx * GTX, y0 = tl.ty * GTY;
+    const int x0 = tl.tx * GTX, y0 = tl.ty * GTY, w = min(GTX, nx - x0), h = min(GTY, ny - y0);
+    constexpr int W = GTX + 2;
+    const int t = threadIdx.x, wid = t >> 5;
     unsigned bad = 0;
-    if (threadIdx.x == 0) sbad = 0;
-    for (int i = threadIdx.x; i < (GTX + 2) * (GTY + 2); i += blockDim.x) {
-        const int x = wrap_any(x0 + i % (GTX + 2) - 1, nx);
-        const int y = wrap_any(y0 + i / (GTX + 2) - 1, ny);
-        float g[9];
-        pull_node<float, float>(fi, x, y, nx, ny, n, g);
-        sp[i] = psi_of_rho<float>(k.rho_ref + sum9(g), k, bad);
+    if (t == 0) sbad = 0;
+    int lx = t & 31, ly = wid;
+    const bool own = wid < GTY && lx < w && ly < h;
+    bool live = own;
+    if (wid >= GTY) {   // the ring: rows -1 and h, then columns -1 and w
+        int r = t - 32 * GTY;
+        live = r < 2 * (w + 2) + 2 * h;
+        if (r < 2 * (w + 2)) {
+            ly = r < w + 2 ? -1 : h;
+            lx = (r < w + 2 ? r : r - (w + 2)) - 1;
+        } else {
+            r -= 2 * (w + 2);
+            lx = r < h ? -1 : w;
+            ly = r < h ? r : r - h;
+        }
+    }
+    const int c = (ly + 1) * W + lx + 1;
+    float g[9];
+    if (live) {
+        const int xs = x0 + lx, ys = y0 + ly;
+        pull_node<float, float>(fi, xs < 0 ? nx - 1 : (xs == nx ? 0 : xs), ys < 0 ? ny - 1 : (ys == ny ? 0 : ys), nx, ny,
+                                n, g);
+        sp[c] = psi_of_rho<float>(k.rho_ref + sum9(g), k, bad);
     }
     __syncthreads();
-    const int tx = threadIdx.x % GTX, ty = threadIdx.x / GTX;
-    const int x = x0 + tx, y = y0 + ty;
-    // Per-node work in FP32 (maxima are exact in any precision; only the
-    // mass and probe-row sums take FP64 arithmetic, the row sums only in the
-    // warps that hold those rows: a warp is one tile row).
-    double rho = 0;
-    float mv = 0.f, dv = 0.f, dr = 0.f, dmax = -1e30f, ndmin = -1e30f;
-    if (x < nx && y < ny) {
-        float g[9];
-        pull_node<float, float>(fi, x, y, nx, ny, n, g);
-        const int W = GTX + 2, c = (ty + 1) * W + tx + 1;
+    float drho = 0.f, mv = 0.f, dv = 0.f, dr = 0.f, dmax = -1e30f, ndmin = -1e30f;
+    const int y = y0 + ly, x = x0 + lx;
+    if (own) {
         Stencil<float> q{sp[c], sp[c + 1], sp[c + W], sp[c - 1], sp[c - W],
                          sp[c + W + 1], sp[c + W - 1], sp[c - W - 1], sp[c - W + 1]};
-        float Fx, Fy, drho, jx, jy;
+        float Fx, Fy, jx, jy;
         force<float>(q, k, Fx, Fy);
         moments<float>(g, drho, jx, jy);
         const float rc = k.rho_ref + drho;
-        rho = double(k.rho_ref) + double(drho);
         const float vx = jx / rc + 0.5f * Fx / rc;
         const float vy = jy / rc + 0.5f * Fy / rc;
         if (!isfinite(drho) || !isfinite(vx) || !isfinite(vy)) bad |= ST_NONFINITE;
         const size_t o = (size_t)I->node_off + (size_t)y * nx + x;
-        if (mode & BO_RHO) rho_out[o] = rho;
+        const bool centre = x == nx / 2 && y == ny / 2, corner = x == 0 && y == 0;
+        if ((mode & BO_RHO) || centre || corner) {
+            const double rho = double(k.rho_ref) + double(drho);
+            if (mode & BO_RHO) rho_out[o] = rho;
+            if (centre) obs[tl.inst].rho_center = rho;
+            if (corner) obs[tl.inst].rho_corner = rho;
+        }
         dv = 1e30f;
         dr = 1e30f;
         if (mode & BO_SNAP) {
@@ -205,35 +249,44 @@ k_observe_batch(const float* __restrict__ f, const BInst* __restrict__ inst, con
         if (isnan(mv)) mv = 1e30f;
         dmax = drho;
         ndmin = -drho;
-        if (x == nx / 2 && y == ny / 2) obs[tl.inst].rho_center = rho;
-        if (x == 0 && y == 0) obs[tl.inst].rho_corner = rho;
     }
-    const bool mid_row = y == ny / 2, row_0 = y == 0;   // uniform over the warp
-    double v[8];
-    v[0] = warp_sum(rho);
-    v[1] = mid_row ? warp_sum(rho) : 0.0;
-    v[2] = row_0 ? warp_sum(rho) : 0.0;
-    v[3] = double(warp_max(mv));
-    v[4] = double(warp_max(dv));
-    v[5] = double(warp_max(dr));
-    v[6] = double(k.rho_ref) + double(warp_max(dmax));
-    v[7] = -(double(k.rho_ref) + double(-warp_max(ndmin)));
-    const unsigned wb = __reduce_or_sync(0xffffffffu, bad);
-    const int wid = threadIdx.x / 32;
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) {
-        for (int j = 0; j < 8; ++j) red[j][wid] = v[j];
-        if (wb) atomicOr(&sbad, wb);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        BPart p;
-        p.sum[0] = p.sum[1] = p.sum[2] = 0;
-        for (int j = 0; j < 5; ++j) p.mx[j] = -1e300;
-        for (int w = 0; w < GTX * GTY / 32; ++w) {
-            for (int j = 0; j < 3; ++j) p.sum[j] += red[j][w];
-            for (int j = 0; j < 5; ++j) p.mx[j] = fmax(p.mx[j], red[3 + j][w]);
+    if (wid < GTY) {   // a warp is one tile row
+        const FPair m = warp_pair_sum(drho);
+        const bool mid_row = y == ny / 2, row_0 = y == 0;
+        const float r[9] = {m.s, m.e, mid_row ? m.s : 0.f, mid_row ? m.e : 0.f, row_0 ? m.s : 0.f, row_0 ? m.e : 0.f,
+                            warp_max(mv), warp_max(dv), warp_max(dr)};
+        const float r9 = warp_max(dmax), r10 = warp_max(ndmin);
+        if ((t & 31) == 0) {
+#pragma unroll
+            for (int j = 0; j < 9; ++j) red[j][wid] = r[j];
+            red[9][wid] = r9;
+            red[10][wid] = r10;
         }
+    }
+    const unsigned wb = __reduce_or_sync(0xffffffffu, bad);
+    if ((t & 31) == 0 && wb) atomicOr(&sbad, wb);
+    __syncthreads();
+    if (t == 0) {
+        FPair m{0.f, 0.f}, mid{0.f, 0.f}, r0{0.f, 0.f};
+        float mx[5] = {0.f, 0.f, 0.f, -1e30f, -1e30f};
+        for (int i = 0; i < h; ++i) {
+            m = pair_add(m, FPair{red[0][i], red[1][i]});
+            mid = pair_add(mid, FPair{red[2][i], red[3][i]});
+            r0 = pair_add(r0, FPair{red[4][i], red[5][i]});
+            for (int j = 0; j < 5; ++j) mx[j] = fmaxf(mx[j], red[6 + j][i]);
+        }
+        // sum of rho = nodes rho_ref + sum of drho
+        const double ref = double(k.rho_ref);
+        const bool has_mid = ny / 2 >= y0 && ny / 2 < y0 + h;
+        BPart p;
+        p.sum[0] = double(w * h) * ref + pair_value(m);
+        p.sum[1] = has_mid ? double(w) * ref + pair_value(mid) : 0.0;
+        p.sum[2] = y0 == 0 ? double(w) * ref + pair_value(r0) : 0.0;
+        p.mx[0] = double(mx[0]);
+        p.mx[1] = double(mx[1]);
+        p.mx[2] = double(mx[2]);
+        p.mx[3] = ref + double(mx[3]);
+        p.mx[4] = -(ref - double(mx[4]));
         p.status = sbad;
         p.pad = 0;
         parts[I->tile_off + tl.ty * I->ntx + tl.tx] = p;
@@ -817,7 +870,7 @@ int step_once(lbm_batch* b)
 int observe(lbm_batch* b, int mode, double tol_v, double tol_rho, double tol_coex, int decide)
 {
     if (b->ntiles) {
-        k_observe_batch<<<b->ntiles, GTX * GTY, 0, b->stream>>>(b->f[b->cur], b->dinst, b->tiles, b->state, b->snap,
+        k_observe_batch<<<b->ntiles, kObsThreads, 0, b->stream>>>(b->f[b->cur], b->dinst, b->tiles, b->state, b->snap,
                                                                b->rho, b->parts, b->obs, mode);
         B_CUDA(cudaGetLastError());
     }
