@@ -261,8 +261,9 @@ int lbm_inject_stage_timeout(lbm_ctx *ctx);
  * strip kernel (nx % 4 == 0).  lbm_set_variant forces one (1 selects the
  * first strip configuration; LBM_E_UNSUPPORTED if the lattice does not
  * allow it); -1 restores the automatic choice: the strip kernel where it
- * applies (for FP32 lattices at least 1024 wide its 256-thread, two-stage
- * configuration; FP64 from 2^21 nodes) and its strips and row chunks can give
+ * applies (FP32: its 256-thread, two-stage configuration, for lattices of
+ * 2^22 nodes and more whose width its 1024 columns cover with at most a
+ * quarter more; FP64: from 2^21 nodes) and its strips and row chunks can give
  * every SM a CTA, else the generic kernel.  lbm_autotune picks by timing. */
 int lbm_get_variant(lbm_ctx *ctx, int *variant);
 int lbm_set_variant(lbm_ctx *ctx, int variant);
@@ -421,14 +422,13 @@ int lbm_batch_profiles(lbm_batch *b, int nb, const lbm_profile_geom *geom_host, 
  *   columns 128: one warp walks a strip; stages 3 or 4 (carry 0), 2 or 3 (carry 1).
  *   columns 256: a 64-thread CTA walks a strip; stages 3, carry 1 only.
  *   columns 512: a 128-thread CTA walks a strip; stages 2 or 3, carry 1 only.
- * Other combinations return LBM_E_INVALID.  Small batches (up to 2^23 running
- * nodes) and narrow lattices step on tiles of at most 256 nodes instead,
- * unless lbm_batch_set_tuning asked for a walk.  lbm_batch_autotune times the
+ * Other combinations return LBM_E_INVALID.  Until a walk is asked for here, a
+ * batch steps on tiles of at most 256 nodes (up to 3 * 2^20 running nodes, and
+ * narrow lattices) or on walks of 32 x 8 tiles.  lbm_batch_autotune times the
  * seven (columns, stages, carry) candidates x rows 32, 64, 128, 256 for
- * trial_steps steps each without advancing the state, and the tiles where
- * they apply, and keeps the fastest (columns .. carry then name the fastest
- * walk, ms_per_step the time of what is kept); any output pointer may be
- * NULL. */
+ * trial_steps steps each without advancing the state, and the tiles, and keeps
+ * the fastest (columns .. carry then name the fastest of the seven,
+ * ms_per_step the time of what is kept); any output pointer may be NULL. */
 int lbm_batch_set_tuning(lbm_batch *b, int columns, int stages, int rows_per_item, int carry);
 int lbm_batch_autotune(lbm_batch *b, int trial_steps, int *columns, int *stages, int *rows_per_item, int *carry,
                        double *ms_per_step);

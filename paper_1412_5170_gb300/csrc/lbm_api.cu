@@ -14,6 +14,7 @@
 #include "lbm_fields.cuh"
 #include "lbm_host.h"
 #include "lbm_kernels.cuh"
+#include "lbm_tilewalk.cuh"
 
 using namespace lbm;
 
@@ -37,6 +38,7 @@ struct lbm_ctx {
     int64_t steps;
     int config;             // 0 = generic kernel, k >= 1 = strip configuration k-1
     TilePlan tile;          // tiles of the generic kernel
+    WalkPlan walk;          // its walks of tiles, for larger FP32 lattices (sx == 0: separate tiles)
     bool inject_timeout = false;   // the next step's first stage waits give up at once
     // Asynchronous host I/O, set up by the first lbm_init_density_async or
     // lbm_read_moments_async: one copy stream per direction, and device
@@ -118,16 +120,26 @@ void launch_generic(lbm_ctx* c, const void* fin, void* fout)
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see k_step_generic
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(c->tile.sx, c->tile.sy);
-    lc.blockDim = dim3(c->tile.threads);
     lc.stream = c->stream;
     lc.attrs = attr;
+    lc.numAttrs = 1;
+    if constexpr (sizeof(T) == sizeof(float)) {
+        if (c->walk.sx) {
+            lc.gridDim = dim3(c->walk.sx, c->walk.sy);
+            lc.blockDim = dim3(kWalkThreads);
+            cudaLaunchKernelEx(&lc, k_step_walk<COLL, FORC>, (const float*)fin, (float*)fout, c->p.nx, c->p.ny,
+                               c->walk.rows, make_coef<float>(c->p), c->status);
+            return;
+        }
+    }
+    lc.gridDim = dim3(c->tile.sx, c->tile.sy);
+    lc.blockDim = dim3(c->tile.threads);
     // FP64 with more tiles than SMs: a plain launch.  A dependent grid's CTAs
     // take whatever slots the running one leaves, several on one SM while
     // others stay empty, which costs the FP64 pipe more than the launch gap
     // (256 x 256: 30.7 us plain, 40.7 us dependent; 64 x 64, one tile per SM:
     // 10.3 plain, 8.1 dependent).
-    lc.numAttrs = c->p.precision == LBM_FP64 && (long long)c->tile.sx * c->tile.sy > sm_count() ? 0 : 1;
+    if (c->p.precision == LBM_FP64 && (long long)c->tile.sx * c->tile.sy > sm_count()) lc.numAttrs = 0;
     cudaLaunchKernelEx(&lc, k_step_generic<T, C, COLL, FORC>, (const T*)fin, (T*)fout, c->p.nx, c->p.ny,
                        make_coef<C>(c->p), c->status);
 }
@@ -146,18 +158,21 @@ void launch_generic_scheme(lbm_ctx* c, const void* fin, void* fout)
 // Without autotuning.  FP64: the generic kernel, whose tiles keep the FP64
 // pipe busier than the strips' few CTAs (1024 x 1024: 356 us a step against
 // 445); from 2^21 nodes the two are close (1024 x 2560: 867 and 922) and the
-// strip kernel stays the automatic choice where it applies.  FP32: the strip
-// kernel where it applies -- for lattices at least 1024 wide the 256-thread,
-// two-stage carried configuration (the fastest measured on large lattices),
-// otherwise the first strip configuration -- unless its strips and row chunks
-// (at least 16 rows each) cannot give every SM a CTA, as on small lattices,
-// where the generic kernel's tiles spread wider; else the generic kernel.
+// strip kernel stays the automatic choice where it applies.  FP32: the
+// 256-thread, two-stage carried strips from 2^22 nodes (2048 x 2048: 69.3 us
+// against 69.6 for the generic kernel's tile walks, 4096 x 4096 217 and 263,
+// but 1536 x 1536 68 and 42, 512 x 4096 58 and 37) where their 1024 columns
+// cover the width with at most a quarter more, else the generic kernel.  Strips also need enough row chunks (at least 16 rows each)
+// to give every SM a CTA.
 int default_config(const lbm_params& p)
 {
     if (!lbm_strip_supported(&p)) return 0;
-    if (p.precision == LBM_FP64 && (long long)p.nx * p.ny < (1 << 21)) return 0;
+    const long long nodes = (long long)p.nx * p.ny;
     int cfg = 1;
-    if (p.precision == LBM_FP32_DEV && p.nx >= 1024) {
+    if (p.precision == LBM_FP64) {
+        if (nodes < (1 << 21)) return 0;
+    } else {
+        if (nodes < (1 << 22) || (p.nx + 1023) / 1024 * 4096LL > 5LL * p.nx) return 0;
         const int n = lbm_strip_config_count(p.precision);
         for (int i = 0; i < n; ++i) {
             const StripConfig sc = lbm_strip_config(p.precision, i);
@@ -400,6 +415,7 @@ int lbm_create(const lbm_params* p, void* cuda_stream, void* workspace_dev, size
     c->cur = 0;
     c->config = default_config(*p);
     c->tile = plan_tiles(p->nx, p->ny, p->precision == LBM_FP64, sm_count());
+    c->walk = p->precision == LBM_FP32_DEV ? plan_walk(p->nx, p->ny, sm_count()) : WalkPlan{0, 0, 0};
     cudaError_t e = cudaMallocHost(&c->hstats, sizeof(DevStats));
     if (e != cudaSuccess) {
         if (c->owns) cudaFree(c->ws);

@@ -22,6 +22,7 @@
 #include "lbm_batch.cuh"
 #include "lbm_fields.cuh"
 #include "lbm_host.h"
+#include "lbm_tilewalk.cuh"
 #include "lbm_warp.cuh"
 
 namespace lbm {
@@ -42,7 +43,7 @@ struct BPart {
 // deviation drho (rho = rho_ref + drho).
 struct __align__(16) Snap { float vx, vy, drho, pad; };
 
-constexpr long long kTileStepNodes = 1 << 23;   // see build_tiles
+constexpr long long kBatchWalkNodes = 3 << 20;   // see build_tiles
 
 constexpr int kBatchWarps = 1;   // warps (independent 128-column walkers) per CTA
 
@@ -129,6 +130,28 @@ k_step_batch_tiles(const float* __restrict__ fin, float* __restrict__ fout, cons
     if (state[tl.inst] != B_RUNNING) return;   // uniform over the CTA
     unsigned bad = 0;
     step_tile<float, float, COLL, FORC>(fin + tl.off, fout + tl.off, tl.nx, tl.ny, tl.x0, tl.y0, tl.w, tl.h, sk, sp, bad);
+    flag_status(bad, &inst_status[tl.inst]);
+}
+
+// The same step as walks of tiles (lbm_tilewalk.cuh): a record's h rows are a
+// chunk its CTA walks down, whatever its height.
+template <int COLL, int FORC>
+__global__ void __launch_bounds__(kWalkThreads, kWalkCtas)
+k_step_batch_walk(const float* __restrict__ fin, float* __restrict__ fout, const BInst* __restrict__ inst,
+                  const BStepTile* __restrict__ tiles, const int* __restrict__ state, unsigned* __restrict__ inst_status)
+{
+    __shared__ WalkPsi sm;
+    __shared__ Coef<float> sk;
+    const BStepTile tl = tiles[blockIdx.x];
+    constexpr int nwords = sizeof(Coef<float>) / sizeof(float);
+    if (threadIdx.x < nwords)
+        reinterpret_cast<float*>(&sk)[threadIdx.x] = reinterpret_cast<const float*>(&inst[tl.inst].k)[threadIdx.x];
+    __syncthreads();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (state[tl.inst] != B_RUNNING) return;   // uniform over the CTA
+    unsigned bad = 0;
+    tile_walk<COLL, FORC>(fin + tl.off, fout + tl.off, tl.nx, tl.ny, tl.x0, tl.w, tl.y0, tl.y0 + tl.h, sk, sm, bad);
     flag_status(bad, &inst_status[tl.inst]);
 }
 
@@ -622,7 +645,8 @@ struct lbm_batch {
     int items_for = 0;           // running instances when the work items were last built
     BStepTile* stiles = nullptr; // tiles of the tiled step
     int nstiles = 0, stiles_cap = 0, stile_threads = 0;
-    bool use_tiles = false;      // the tiled step instead of the walks
+    bool use_tiles = false;      // the tiled step instead of the strip walks
+    bool tile_walks = false;     // its records are chunks to walk
     bool allow_tiles = true;     // false once a walk was asked for (lbm_batch_set_tuning) or timed faster
     int* state = nullptr;        // device
     int* fail = nullptr;         // device
@@ -680,32 +704,43 @@ int batch_sms()
     return nsm;
 }
 
-// Tiles of the running instances for the tiled step, and whether it is used:
-// up to 2^23 nodes (64 instances of the sweep, 7.5 M nodes: 146 us a step
-// against the walk's 178; 256 instances, 25 M nodes, 484 against 462), and
-// for narrow lattices at any size (where whole strips would hold twice the
-// nodes; 200 slabs of 8 x 128: 5.9 us against 72.7).
+// Records of the running instances for the tiled step, which a batch takes
+// unless a strip walk was asked for or timed faster: separate tiles below
+// 3 * 2^20 running nodes or for narrow lattices, walks of tiles from there.
+// Per step, one-warp strip walk / separate tiles / walks of tiles: 24 slabs of
+// 8 x 128 20.6 / 2.5 / 4.7 us, 2.1 M nodes in 64 x 64 lattices 95 / 44 / 43,
+// sweep instances of 3.5 M nodes 88 / 69 / 64, 7.5 M 178 / 146 / 129, 26.6 M
+// 490 / 508 / 429.
 int build_tiles(lbm_batch* b, const int* host_state)
 {
     const int nsm = batch_sms();
-    long long nodes = 0, padded = 0;   // nodes, and nodes of whole 128-column strips
+    long long nodes = 0, tiles8 = 0;   // nodes, and 32 x 8 tiles
     for (int i = 0; i < b->n; ++i) {
         if (host_state && host_state[i] != B_RUNNING) continue;
         const BInst& I = b->hinst[i];
         nodes += (long long)I.nx * I.ny;
-        padded += (long long)((I.nx + 127) / 128 * 128) * I.ny;
+        tiles8 += (long long)((I.nx + 31) / 32) * ((I.ny + 7) / 8);
     }
-    b->use_tiles = b->allow_tiles && (nodes <= kTileStepNodes || padded >= 2 * nodes);
+    b->use_tiles = b->allow_tiles;
+    b->tile_walks = nodes >= kBatchWalkNodes && tiles8 * 256 < 2 * nodes;
     b->nstiles = 0;
     if (!b->use_tiles || nodes == 0) return LBM_OK;
-    // two tiles per SM where the batch is that small, 256 nodes at most (smaller ones cost more ring:
-    // 146, 163 and 213 us a step at 256, 128 and 64 nodes on 7.5 M nodes)
+    // separate tiles: two per SM where the batch is that small, 256 nodes at most (smaller ones cost more
+    // ring: 146, 163 and 213 us a step at 256, 128 and 64 nodes on 7.5 M nodes).  Walks: chunks of at most
+    // 64 rows (25 M nodes: 429 us at 80 rows, 439 at 160, 469 at 320)
     const int want = (int)std::min<long long>(256, std::max<long long>(32, nodes / (2 * nsm)));
+    const int chunk = 8 * (int)std::min<long long>(8, std::max<long long>(1, tiles8 / (16LL * nsm)));
     std::vector<BStepTile> t;
-    b->stile_threads = 0;
+    b->stile_threads = b->tile_walks ? kWalkThreads : 0;
     for (int i = 0; i < b->n; ++i) {
         if (host_state && host_state[i] != B_RUNNING) continue;
         const BInst& I = b->hinst[i];
+        if (b->tile_walks) {
+            for (int y = 0; y < I.ny; y += chunk)
+                for (int x = 0; x < I.nx; x += kWalkW)
+                    t.push_back(BStepTile{I.off, i, I.nx, I.ny, x, y, std::min(kWalkW, I.nx - x), std::min(chunk, I.ny - y), 0});
+            continue;
+        }
         const int sx = (I.nx + 31) / 32, w = (I.nx + sx - 1) / sx;
         const int h0 = std::min(32, std::max(1, want / w)), sy = (I.ny + h0 - 1) / h0, h = (I.ny + sy - 1) / sy;
         b->stile_threads = std::max(b->stile_threads, 32 * ((w * h + 31) / 32 + (2 * (w + 2) + 2 * h + 31) / 32));
@@ -783,7 +818,8 @@ int launch_tiles(lbm_batch* b, const float* fin, float* fout)
 {
     cudaFuncAttributes fa;   // loads the kernel before any graph capture
     static const cudaError_t loaded = cudaFuncGetAttributes(&fa, k_step_batch_tiles<COLL, FORC>);
-    if (loaded != cudaSuccess) return LBM_E_CUDA;
+    static const cudaError_t loaded_walk = cudaFuncGetAttributes(&fa, k_step_batch_walk<COLL, FORC>);
+    if (loaded != cudaSuccess || loaded_walk != cudaSuccess) return LBM_E_CUDA;
     if (b->nstiles == 0) return LBM_OK;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see k_step_batch_tiles
@@ -794,7 +830,8 @@ int launch_tiles(lbm_batch* b, const float* fin, float* fout)
     lc.stream = b->stream;
     lc.attrs = attr;
     lc.numAttrs = 1;
-    return cudaLaunchKernelEx(&lc, k_step_batch_tiles<COLL, FORC>, fin, fout, (const BInst*)b->dinst,
+    auto kern = b->tile_walks ? k_step_batch_walk<COLL, FORC> : k_step_batch_tiles<COLL, FORC>;
+    return cudaLaunchKernelEx(&lc, kern, fin, fout, (const BInst*)b->dinst,
                               (const BStepTile*)b->stiles, (const int*)b->state, b->status) == cudaSuccess
                ? LBM_OK : LBM_E_CUDA;
 }

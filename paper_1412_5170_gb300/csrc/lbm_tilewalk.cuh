@@ -1,0 +1,118 @@
+// lbm_tilewalk.cuh -- the FP32 step as a walk of 32 x 8 tiles down a strip of
+// 32 columns, one node per thread, for lattices of any width (plain 32-bit
+// loads: no alignment of rows is needed, which the strip walks' 16-byte
+// copies take for granted).
+//
+// Eight warps hold the tile's rows, two more the nodes to its left, right and
+// below whose psi the force needs; the psi above is the last row of the tile
+// before.  Each thread loads its nine pulled values of the next tile before
+// it collides the current one, so a CTA always has a tile of loads in flight;
+// a grid of separate tiles (the generic step) waits out the memory latency
+// once per tile instead, at 45 nodes/ns whatever the size.  One barrier per
+// tile: psi is double-buffered.  Per step, separate tiles and this (MRT):
+// 384 x 384 6.0 and 4.6 us, 1023 x 1021 23.1 and 19.5, 2047 x 2049 85.7 and
+// 69.6, 4096 x 4096 335 and 263 (the strip walks 217); 256 sweep instances
+// 508 and 429 (the one-warp strip walk 490).  What bounds it now is issue (55
+// % of the slots at 4096 x 4096) and the latency left per tile; HBM is at 0.67.
+#pragma once
+#include <cuda_runtime.h>
+
+#include "lbm_kernels.cuh"
+
+namespace lbm {
+
+constexpr int kWalkW = 32, kWalkH = 8, kWalkThreads = 32 * (kWalkH + 2);
+constexpr int kWalkRow = kWalkW + 2;
+constexpr int kWalkCtas = 4;   // per SM: 48 registers a thread
+
+struct WalkPsi { float p[2][(kWalkH + 2) * kWalkRow]; };
+
+// Columns [x0, x0 + w) with w <= 32, rows [y0, y1) of an nx x ny lattice; all
+// kWalkThreads threads call it, after their griddepcontrol.wait.
+template <int COLL, int FORC>
+__device__ __forceinline__ void tile_walk(const float* __restrict__ fin, float* __restrict__ fout, int nx, int ny, int x0,
+                                          int w, int y0, int y1, const Coef<float>& k, WalkPsi& sm, unsigned& bad)
+{
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    const size_t n = (size_t)nx * ny;
+    const bool mine = wid < kWalkH;
+    // ring threads: the row below (w + 2 nodes from column -1 on), then the columns -1 and w of the tile's rows
+    const int r = t - 32 * kWalkH;
+    const bool below = !mine && r < w + 2;
+    const int side = r - (w + 2);   // 0 .. 15: row side / 2 of the left (even) or right (odd) column
+    const int lx = mine ? lane : (below ? r - 1 : (side & 1 ? w : -1));
+    const bool used = mine ? lane < w : (below || side < 2 * kWalkH);
+    const int xs = x0 + lx < 0 ? nx - 1 : (x0 + lx >= nx ? 0 : x0 + lx);   // idle lanes of a ragged strip: any column
+    const int xm = dec1(xs, nx), xp = inc1(xs, nx);
+    // row of this thread's node in a tile of h rows
+    auto row_of = [&](int h) { return mine ? wid : (below ? h : side >> 1); };
+    auto live_in = [&](int h) { return used && (below || row_of(h) < h); };
+    auto load = [&](int y, float (&g)[9]) {
+        const int ys = y < 0 ? ny - 1 : (y >= ny ? y - ny : y);
+        const size_t r0 = (size_t)ys * nx, rm = (size_t)dec1(ys, ny) * nx, rp = (size_t)inc1(ys, ny) * nx;
+        g[0] = fin[0 * n + r0 + xs];
+        g[1] = fin[1 * n + r0 + xm];
+        g[2] = fin[2 * n + rm + xs];
+        g[3] = fin[3 * n + r0 + xp];
+        g[4] = fin[4 * n + rp + xs];
+        g[5] = fin[5 * n + rm + xm];
+        g[6] = fin[6 * n + rm + xp];
+        g[7] = fin[7 * n + rp + xp];
+        g[8] = fin[8 * n + rp + xm];
+    };
+
+    float gA[9], gB[9];
+    // the row above the first tile
+    if (below) {
+        load(y0 - 1, gA);
+        sm.p[0][lx + 1] = psi_of_rho<float>(k.rho_ref + sum9(gA), k, bad);
+    }
+    int h = min(kWalkH, y1 - y0);
+    if (live_in(h)) load(y0 + row_of(h), gA);
+
+    auto body = [&](int y, int buf, float (&g)[9], float (&gn)[9]) {
+        float* p = sm.p[buf];
+        const int ly = row_of(h);
+        if (live_in(h)) p[(ly + 1) * kWalkRow + lx + 1] = psi_of_rho<float>(k.rho_ref + sum9(g), k, bad);
+        const int hn = min(kWalkH, y1 - y - h);
+        if (hn > 0 && live_in(hn)) load(y + h + row_of(hn), gn);   // the next tile, in flight from here
+        __syncthreads();
+        if (mine && lane < w && ly < h) {
+            const int c = (ly + 1) * kWalkRow + lane + 1;
+            Stencil<float> q{p[c], p[c + 1], p[c + kWalkRow], p[c - 1], p[c - kWalkRow],
+                             p[c + kWalkRow + 1], p[c + kWalkRow - 1], p[c - kWalkRow - 1], p[c - kWalkRow + 1]};
+            float Fx, Fy, vx, vy, rho;
+            force<float>(q, k, Fx, Fy);
+            collide<float, COLL, FORC>(g, Fx, Fy, k, vx, vy, rho, q.c);
+            if (!isfinite(g[0])) bad |= ST_NONFINITE;   // g0 closes on all others
+            float* o = fout + (size_t)(y + ly) * nx + x0 + lane;
+#pragma unroll
+            for (int a = 0; a < 9; ++a) o[a * n] = g[a];
+        } else if (below) {
+            sm.p[buf ^ 1][lx + 1] = p[h * kWalkRow + lx + 1];   // the last row's psi: above the next tile
+        }
+        h = hn;
+    };
+    for (int y = y0; y < y1; y += 2 * kWalkH) {
+        body(y, 0, gA, gB);
+        if (y + kWalkH < y1) body(y + kWalkH, 1, gB, gA);
+    }
+}
+
+// One lattice: grid (32-column strips, chunks of `rows` rows).
+template <int COLL, int FORC>
+__global__ void __launch_bounds__(kWalkThreads, kWalkCtas)
+k_step_walk(const float* __restrict__ fin, float* __restrict__ fout, int nx, int ny, int rows, Coef<float> k,
+            unsigned* __restrict__ status)
+{
+    __shared__ WalkPsi sm;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int x0 = blockIdx.x * kWalkW;
+    const int y0 = blockIdx.y * rows;
+    unsigned bad = 0;
+    tile_walk<COLL, FORC>(fin, fout, nx, ny, x0, min(kWalkW, nx - x0), y0, min(y0 + rows, ny), k, sm, bad);
+    flag_status(bad, status);
+}
+
+}  // namespace lbm

@@ -51,3 +51,20 @@ def test_tiles_follow_the_running_instances(lbm):
     assert state[3] == lbm.FAILED and code[3] in (lbm.E_NONFINITE, lbm.E_EOS_DOMAIN)
     assert (state[:3] == lbm.CONVERGED).all() and steps[3] < steps[:3].min() + 20000
     assert np.ptp(obs["rho_row_mid"][:3]) < 1e-6 and (obs["rho_row_mid"][:3] > 5 * obs["rho_row0"][:3]).all()
+
+
+def test_large_batches_walk_tiles(lbm):
+    """More than 3 * 2^20 nodes: chunks of tiles, against the one-warp walk."""
+    inst = [dict(nx=512, ny=512, kind="droplet", T_over_Tc=0.8, tau=0.9, A=-0.304, K=1.0, size=100.0, seed=i) for i in range(12)]
+    inst += [dict(nx=nx, ny=ny, kind="slab", T_over_Tc=0.75, tau=0.7, A=-0.304, K=0.5, size=ny / 4, seed=50 + ny)
+             for nx, ny in ((4, 9), (36, 65), (516, 331))]
+    out = []
+    for walk in (False, True):
+        with lbm.Batch(inst, collision="mrt") as b:
+            if walk:
+                b.set_tuning(128, 3, 32)
+            b.init()
+            b.step(20)
+            out.append([b.read_density(i) for i in range(len(inst))])
+    for x, y in zip(*out):
+        assert (np.abs(x - y) / y).max() < 2e-6

@@ -33,3 +33,23 @@ def test_tiles(lbm, nx, ny, coll, forc, precision):
         assert np.abs(f - ref).max() < 1e-12 * np.abs(ref).max()
     else:
         assert (np.abs(f.sum(0) - ref.sum(0)) / ref.sum(0)).max() < 2e-5
+
+
+# 2^17 nodes and more: walks of 32 x 8 tiles; ragged last strips and chunks,
+# strips of one column (1057 = 33 * 32 + 1), fewer columns than a strip
+@pytest.mark.parametrize("coll,forc", [("mrt", "guo"), ("bgk", "guo"), ("bgk", "edm"), ("bgk", "sc"), ("bgk", "li")])
+@pytest.mark.parametrize("nx,ny", [(379, 361), (1057, 129), (31, 4231), (4231, 33)])
+def test_tile_walks(lbm, nx, ny, coll, forc):
+    rv, rl = lbm.maxwell(0.8)
+    rho0 = synth.density_field(nx, ny, "droplet", rl, rv, min(nx, ny) / 4, seed=5)
+    A, sigma = (0.0, 0.105) if forc == "li" else (-0.304, 0.0)
+    p = lbm.make_params(nx, ny, 0.8, 0.9, A, 1.0, coll, forc, "fp32", sigma=sigma, **MRT)
+    with lbm.Lattice(p) as lat:
+        assert lat.config == 0
+        lat.init_density(rho0)
+        lat.step(10)
+        f, st = lat.read_populations(), lat.stats()
+    ref, ost = oracle.run(oracle.params(nx, ny, 0.8, 0.9, A, 1.0, coll, forc, sigma=sigma, **MRT), oracle.init_rest(rho0), 10)
+    assert ost == 0 and st["status"] == 0
+    assert (np.abs(f.sum(0) - ref.sum(0)) / ref.sum(0)).max() < 2e-5
+    assert np.abs(f - ref).max() < 2e-5 * np.abs(ref).max()
