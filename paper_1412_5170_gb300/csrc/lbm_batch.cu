@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(kWalkThreads, kWalkCtas)
 k_step_batch_walk(const float* __restrict__ fin, float* __restrict__ fout, const BInst* __restrict__ inst,
                   const BStepTile* __restrict__ tiles, const int* __restrict__ state, unsigned* __restrict__ inst_status)
 {
-    __shared__ WalkPsi sm;
+    __shared__ WalkPsi<float> sm;
     __shared__ Coef<float> sk;
     const BStepTile tl = tiles[blockIdx.x];
     constexpr int nwords = sizeof(Coef<float>) / sizeof(float);
@@ -151,7 +151,8 @@ k_step_batch_walk(const float* __restrict__ fin, float* __restrict__ fout, const
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (state[tl.inst] != B_RUNNING) return;   // uniform over the CTA
     unsigned bad = 0;
-    tile_walk<COLL, FORC>(fin + tl.off, fout + tl.off, tl.nx, tl.ny, tl.x0, tl.w, tl.y0, tl.y0 + tl.h, sk, sm, bad);
+    StepNode<float, float, COLL, FORC> node{fout + tl.off, tl.nx, (size_t)tl.nx * tl.ny};
+    tile_walk<float, float>(fin + tl.off, tl.nx, tl.ny, tl.x0, tl.w, tl.y0, tl.y0 + tl.h, sk, sm, bad, node);
     flag_status(bad, &inst_status[tl.inst]);
 }
 

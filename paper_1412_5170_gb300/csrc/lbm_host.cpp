@@ -243,22 +243,20 @@ TilePlan plan_tiles(int nx, int ny, bool fp64, int nsm)
     return best;
 }
 
-// From 2^17 nodes: 384 x 384 4.7-5.1 us a step against 6.0 on separate tiles,
-// 257 x 259 4.1 against 3.4.  Chunks are whole tiles of 8 rows; of all chunk
-// heights the one is taken whose waves of CTAs (four per SM are resident)
-// cost least, a chunk of m tiles counting as m + 1/2 for its first loads.  A
-// single wave counts a tenth more: its CTAs all start and end together
-// (2047 x 2049: 75 us in one wave of 576, 70 in two of 608).
-WalkPlan plan_walk(int nx, int ny, int nsm)
+// Chunks are whole tiles of 8 rows; of all chunk heights the one is taken
+// whose waves of CTAs cost least, a chunk of m tiles counting as m + 1/2 for
+// its first loads.  A single wave counts a tenth more: its CTAs all start and
+// end together (FP32 step, 2047 x 2049: 75 us in one wave of 576, 70 in two of
+// 608).
+WalkPlan plan_walk(int nx, int ny, int nsm, int ctas)
 {
-    if ((int64_t)nx * ny < (1 << 17)) return WalkPlan{0, 0, 0};
     const int sx = (nx + 31) / 32, tiles = (ny + 7) / 8;
     WalkPlan best{0, 0, 0};
     double best_cost = 0;
-    for (int m = 1; m <= tiles && m <= 512; ++m) {
+    for (int m = 1; m <= tiles && (m <= 512 || best.sx == 0); ++m) {
         const int sy = (tiles + m - 1) / m;
         if (sy > 65535) continue;
-        const double f = double(sx) * sy / (4.0 * nsm);
+        const double f = double(sx) * sy / (double(ctas) * nsm);
         const double cost = (f <= 1 ? 1.1 : f + 0.5 / f) * (m + 0.5);
         if (best.sx == 0 || cost < best_cost) {
             best = WalkPlan{sx, sy, 8 * m};

@@ -26,11 +26,10 @@ int lbm_validate_preset(int nx, int ny, int kind, double size, double width, int
 // one CTA of `threads` threads each.
 struct TilePlan { int sx, sy, threads; };
 TilePlan plan_tiles(int nx, int ny, bool fp64, int nsm);
-// Strips of 32 columns and chunks of `rows` rows of the FP32 walks of tiles
-// (lbm_tilewalk.cuh), one CTA each; sx = 0 where separate tiles are the
-// better choice.
+// Strips of 32 columns and chunks of `rows` rows of the walks of tiles
+// (lbm_tilewalk.cuh), one CTA each, `ctas` of which an SM holds.
 struct WalkPlan { int sx, sy, rows; };
-WalkPlan plan_walk(int nx, int ny, int nsm);
+WalkPlan plan_walk(int nx, int ny, int nsm, int ctas);
 
 // Polls of a bounded stage wait (mbarrier try_wait) before the staged kernels
 // declare a row copy stuck, flag a timeout, drain and return.

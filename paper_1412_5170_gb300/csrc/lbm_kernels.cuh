@@ -412,14 +412,12 @@ __global__ void k_plane_convert(T* __restrict__ fs, double* __restrict__ plane, 
     }
 }
 
-// The observation with the strip walk (lbm_observe.cu), for lattices the strip
-// kernel supports (nx % 4 == 0): mode as k_observe; with OBS_REDUCE the per-CTA
-// partials (parts, at least as many as the generic observation's tiles) are
-// reduced in the same launch by the last CTA to finish, in a fixed order,
+// The observation of a lattice (lbm_observe.cu): mode as k_observe; with
+// OBS_REDUCE the per-CTA partials (parts, at least as many as 32 x 8 tiles)
+// are reduced in the same launch by the last CTA to finish, in a fixed order,
 // into ds (ticket: a device counter that is 0 between launches).  vsnap holds
 // VSnap<C> of the precision's compute type.
-int observe_strip_launch(const lbm_params* p, const void* f, int mode, double* rho, double* vx, double* vy,
-                         void* vsnap, Partial* parts, unsigned* ticket, DevStats* ds, const unsigned* status,
-                         cudaStream_t s);
+int observe_launch(const lbm_params* p, const void* f, int mode, double* rho, double* vx, double* vy, void* vsnap,
+                   Partial* parts, unsigned* ticket, DevStats* ds, const unsigned* status, int nsm, cudaStream_t s);
 
 }  // namespace lbm

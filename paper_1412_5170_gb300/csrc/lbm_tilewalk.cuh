@@ -25,13 +25,38 @@ constexpr int kWalkW = 32, kWalkH = 8, kWalkThreads = 32 * (kWalkH + 2);
 constexpr int kWalkRow = kWalkW + 2;
 constexpr int kWalkCtas = 4;   // per SM: 48 registers a thread
 
-struct WalkPsi { float p[2][(kWalkH + 2) * kWalkRow]; };
+template <typename C>
+struct WalkPsi { C p[2][(kWalkH + 2) * kWalkRow]; };
 
-// Columns [x0, x0 + w) with w <= 32, rows [y0, y1) of an nx x ny lattice; all
-// kWalkThreads threads call it, after their griddepcontrol.wait.
-template <int COLL, int FORC>
-__device__ __forceinline__ void tile_walk(const float* __restrict__ fin, float* __restrict__ fout, int nx, int ny, int x0,
-                                          int w, int y0, int y1, const Coef<float>& k, WalkPsi& sm, unsigned& bad)
+// The time step of one node (x, y) from its pulled populations and the psi
+// stencil around it.
+template <typename T, typename C, int COLL, int FORC>
+struct StepNode {
+    T* __restrict__ fout;
+    int nx;
+    size_t n;
+    __device__ __forceinline__ void operator()(int y, int x, C (&g)[9], const Stencil<C>& q, const Coef<C>& k,
+                                               unsigned& bad) const
+    {
+        C Fx, Fy, vx, vy, rho;
+        force<C>(q, k, Fx, Fy);
+        collide<C, COLL, FORC>(g, Fx, Fy, k, vx, vy, rho, q.c);
+        if constexpr (sizeof(C) == sizeof(float)) {
+            if (!isfinite(g[0])) bad |= ST_NONFINITE;   // g0 closes on all others
+        } else {
+            bad |= finite_bits<C>(g);
+        }
+        T* o = fout + (size_t)y * nx + x;
+#pragma unroll
+        for (int a = 0; a < 9; ++a) o[a * n] = T(g[a]);
+    }
+};
+
+// Columns [x0, x0 + w) with w <= 32, rows [y0, y1) of an nx x ny lattice, each
+// node handed to `node` once; all kWalkThreads threads call it.
+template <typename T, typename C, class Node>
+__device__ __forceinline__ void tile_walk(const T* __restrict__ fin, int nx, int ny, int x0, int w, int y0, int y1,
+                                          const Coef<C>& k, WalkPsi<C>& sm, unsigned& bad, Node& node)
 {
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     const size_t n = (size_t)nx * ny;
@@ -47,47 +72,41 @@ __device__ __forceinline__ void tile_walk(const float* __restrict__ fin, float* 
     // row of this thread's node in a tile of h rows
     auto row_of = [&](int h) { return mine ? wid : (below ? h : side >> 1); };
     auto live_in = [&](int h) { return used && (below || row_of(h) < h); };
-    auto load = [&](int y, float (&g)[9]) {
+    auto load = [&](int y, C (&g)[9]) {
         const int ys = y < 0 ? ny - 1 : (y >= ny ? y - ny : y);
         const size_t r0 = (size_t)ys * nx, rm = (size_t)dec1(ys, ny) * nx, rp = (size_t)inc1(ys, ny) * nx;
-        g[0] = fin[0 * n + r0 + xs];
-        g[1] = fin[1 * n + r0 + xm];
-        g[2] = fin[2 * n + rm + xs];
-        g[3] = fin[3 * n + r0 + xp];
-        g[4] = fin[4 * n + rp + xs];
-        g[5] = fin[5 * n + rm + xm];
-        g[6] = fin[6 * n + rm + xp];
-        g[7] = fin[7 * n + rp + xp];
-        g[8] = fin[8 * n + rp + xm];
+        g[0] = C(fin[0 * n + r0 + xs]);
+        g[1] = C(fin[1 * n + r0 + xm]);
+        g[2] = C(fin[2 * n + rm + xs]);
+        g[3] = C(fin[3 * n + r0 + xp]);
+        g[4] = C(fin[4 * n + rp + xs]);
+        g[5] = C(fin[5 * n + rm + xm]);
+        g[6] = C(fin[6 * n + rm + xp]);
+        g[7] = C(fin[7 * n + rp + xp]);
+        g[8] = C(fin[8 * n + rp + xm]);
     };
 
-    float gA[9], gB[9];
+    C gA[9], gB[9];
     // the row above the first tile
     if (below) {
         load(y0 - 1, gA);
-        sm.p[0][lx + 1] = psi_of_rho<float>(k.rho_ref + sum9(gA), k, bad);
+        sm.p[0][lx + 1] = psi_of_rho<C>(k.rho_ref + sum9(gA), k, bad);
     }
     int h = min(kWalkH, y1 - y0);
     if (live_in(h)) load(y0 + row_of(h), gA);
 
-    auto body = [&](int y, int buf, float (&g)[9], float (&gn)[9]) {
-        float* p = sm.p[buf];
+    auto body = [&](int y, int buf, C (&g)[9], C (&gn)[9]) {
+        C* p = sm.p[buf];
         const int ly = row_of(h);
-        if (live_in(h)) p[(ly + 1) * kWalkRow + lx + 1] = psi_of_rho<float>(k.rho_ref + sum9(g), k, bad);
+        if (live_in(h)) p[(ly + 1) * kWalkRow + lx + 1] = psi_of_rho<C>(k.rho_ref + sum9(g), k, bad);
         const int hn = min(kWalkH, y1 - y - h);
         if (hn > 0 && live_in(hn)) load(y + h + row_of(hn), gn);   // the next tile, in flight from here
         __syncthreads();
         if (mine && lane < w && ly < h) {
             const int c = (ly + 1) * kWalkRow + lane + 1;
-            Stencil<float> q{p[c], p[c + 1], p[c + kWalkRow], p[c - 1], p[c - kWalkRow],
-                             p[c + kWalkRow + 1], p[c + kWalkRow - 1], p[c - kWalkRow - 1], p[c - kWalkRow + 1]};
-            float Fx, Fy, vx, vy, rho;
-            force<float>(q, k, Fx, Fy);
-            collide<float, COLL, FORC>(g, Fx, Fy, k, vx, vy, rho, q.c);
-            if (!isfinite(g[0])) bad |= ST_NONFINITE;   // g0 closes on all others
-            float* o = fout + (size_t)(y + ly) * nx + x0 + lane;
-#pragma unroll
-            for (int a = 0; a < 9; ++a) o[a * n] = g[a];
+            const Stencil<C> q{p[c], p[c + 1], p[c + kWalkRow], p[c - 1], p[c - kWalkRow],
+                               p[c + kWalkRow + 1], p[c + kWalkRow - 1], p[c - kWalkRow - 1], p[c - kWalkRow + 1]};
+            node(y + ly, x0 + lane, g, q, k, bad);
         } else if (below) {
             sm.p[buf ^ 1][lx + 1] = p[h * kWalkRow + lx + 1];   // the last row's psi: above the next tile
         }
@@ -105,13 +124,14 @@ __global__ void __launch_bounds__(kWalkThreads, kWalkCtas)
 k_step_walk(const float* __restrict__ fin, float* __restrict__ fout, int nx, int ny, int rows, Coef<float> k,
             unsigned* __restrict__ status)
 {
-    __shared__ WalkPsi sm;
+    __shared__ WalkPsi<float> sm;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int x0 = blockIdx.x * kWalkW;
     const int y0 = blockIdx.y * rows;
     unsigned bad = 0;
-    tile_walk<COLL, FORC>(fin, fout, nx, ny, x0, min(kWalkW, nx - x0), y0, min(y0 + rows, ny), k, sm, bad);
+    StepNode<float, float, COLL, FORC> node{fout, nx, (size_t)nx * ny};
+    tile_walk<float, float>(fin, nx, ny, x0, min(kWalkW, nx - x0), y0, min(y0 + rows, ny), k, sm, bad, node);
     flag_status(bad, status);
 }
 

@@ -166,9 +166,9 @@ def check(status, what=""):
 
 
 def strip_observation(p: lbm_params) -> bool:
-    """Whether lbm_stats observes p's lattice with the strip walk (one launch,
-    reduction included): the lattices the strip kernel takes, nx % 4 == 0."""
-    return p.nx >= 4 and p.nx % 4 == 0
+    """Whether lbm_stats observes p's lattice in one launch, reduction
+    included: every lattice (walks of tiles down strips of 32 columns)."""
+    return p.nx >= 1 and p.ny >= 1
 
 
 def fma_peak(precision: str = "fp64") -> float:
