@@ -152,27 +152,36 @@ void launch_generic_scheme(lbm_ctx* c, const void* fin, void* fout)
 // Without autotuning.  FP64: the generic kernel, whose tiles keep the FP64
 // pipe busier than the strips' few CTAs (1024 x 1024: 356 us a step against
 // 445); from 2^21 nodes the two are close (1024 x 2560: 867 and 922) and the
-// strip kernel stays the automatic choice where it applies.  FP32: the
-// 256-thread, two-stage carried strips from 2^22 nodes (2048 x 2048: 69.3 us
-// against 69.6 for the generic kernel's tile walks, 4096 x 4096 217 and 263,
-// but 1536 x 1536 68 and 42, 512 x 4096 58 and 37) where their 1024 columns
-// cover the width with at most a quarter more, else the generic kernel.  Strips also need enough row chunks (at least 16 rows each)
-// to give every SM a CTA.
+// strip kernel stays the automatic choice where it applies.
+// FP32 below 2^22 nodes: the generic kernel (1536 x 1536 42 us against 68 for
+// 1024-column strips, 512 x 4096 37 and 58).  From there the two-stage carried
+// strips of 1024 or 512 columns, the wider one whose last strip wastes at most
+// a sixteenth of the width: 4096 x 4096 211.5 us with 1024 columns, 252.6
+// with 512 and 252 with the generic kernel; 3072 x 3072 125 and 147 (generic
+// 149); 2560 x 4096 162 and 148 (generic 162).  (2048 columns, 208.5 us at
+// 4096 x 4096, take a whole SM per CTA: three lattices stepping on streams of
+// their own then need 4 % longer than with 1024.)
+// Strips also need enough row chunks (at least 16 rows each) to give every SM
+// a CTA.
 int default_config(const lbm_params& p)
 {
     if (!lbm_strip_supported(&p)) return 0;
     const long long nodes = (long long)p.nx * p.ny;
-    int cfg = 1;
+    int cfg = 0;
     if (p.precision == LBM_FP64) {
-        if (nodes < (1 << 21)) return 0;
-    } else {
-        if (nodes < (1 << 22) || (p.nx + 1023) / 1024 * 4096LL > 5LL * p.nx) return 0;
+        if (nodes >= (1 << 21)) cfg = 1;
+    } else if (nodes >= (1 << 22)) {
         const int n = lbm_strip_config_count(p.precision);
-        for (int i = 0; i < n; ++i) {
-            const StripConfig sc = lbm_strip_config(p.precision, i);
-            if (sc.threads == 256 && sc.stages == 2) { cfg = i + 1; break; }
+        for (int threads = 256; threads >= 128 && cfg == 0; threads /= 2) {
+            const long long width = 4LL * threads, padded = (p.nx + width - 1) / width * width;
+            if (16 * padded > 17LL * p.nx) continue;
+            for (int i = 0; i < n; ++i) {   // the last of that shape (256 threads: seam copies one per lane)
+                const StripConfig sc = lbm_strip_config(p.precision, i);
+                if (sc.threads == threads && sc.stages == 2 && sc.warp == 4) cfg = i + 1;
+            }
         }
     }
+    if (cfg == 0) return 0;
     const StripConfig sc = lbm_strip_config(p.precision, cfg - 1);
     const long long width = 4LL * sc.threads;
     const long long strips = (p.nx + width - 1) / width;
