@@ -352,41 +352,29 @@ k_reduce_final(const Partial* __restrict__ parts, int nparts, int nx, DevStats* 
 // user-facing form) and the stored pull-convention deviations
 // f*_a(x, t-1) - w_a rho_ref = f_a(x + e_a, t) - w_a rho_ref.
 // ---------------------------------------------------------------------------
+// A start at rest, f_a = w_a rho0, as stored values in one pass: the thread of
+// a node writes its population of direction a to the node that stores it,
+// x - e_a (a warp's stores stay contiguous).  FP32: w_a float(rho0 - rho_ref),
+// so one FP64 subtraction a node.  Bound by HBM, 8 B read and 36 B (FP64 72 B)
+// written per node; in two passes through an array of deviations, each node
+// found by a 64-bit division, 4096 x 4096 took 200 us in FP32, now 130.
 template <typename T>
-__global__ void k_init_rest(const double* __restrict__ rho0, T* __restrict__ fs, int nx, int ny, double rho_ref)
+__global__ void __launch_bounds__(256)
+k_init_rest(const double* __restrict__ rho0, T* __restrict__ fs, int nx, int ny, double rho_ref)
 {
     const size_t n = (size_t)nx * ny;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const int x = int(i % nx), y = int(i / nx);
+    const int x = blockIdx.x * 256 + threadIdx.x;
+    if (x >= nx) return;
+    const int xl = dec1(x, nx), xr = inc1(x, nx);
+    for (int y = blockIdx.y; y < ny; y += gridDim.y) {
+        const size_t row = (size_t)y * nx, rd = (size_t)dec1(y, ny) * nx, ru = (size_t)inc1(y, ny) * nx;
+        const double r = rho0[row + x];
+        const float d = float(r - rho_ref);
 #pragma unroll
         for (int a = 0; a < 9; ++a) {
-            const int xs = ex(a) > 0 ? inc1(x, nx) : (ex(a) < 0 ? dec1(x, nx) : x);
-            const int ys = ey(a) > 0 ? inc1(y, ny) : (ey(a) < 0 ? dec1(y, ny) : y);
-            const double w = wt<double>(a);
-            fs[a * n + i] = T(w * rho0[(size_t)ys * nx + xs] - w * rho_ref);
-        }
-    }
-}
-
-// FP32-deviation initial state in two passes, off the FP64 pipe: the density
-// deviation of every node once, dev = float(rho0 - rho_ref), then
-// g_a(x) = w_a dev(x + e_a) (the stored f*_a(x) of a start at rest).
-static __global__ void k_init_dev_f32(const double* __restrict__ rho0, float* __restrict__ dev, size_t n, double rho_ref)
-{
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        dev[i] = float(rho0[i] - rho_ref);
-}
-
-static __global__ void k_init_rest_f32(const float* __restrict__ dev, float* __restrict__ fs, int nx, int ny)
-{
-    const size_t n = (size_t)nx * ny;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const int x = int(i % nx), y = int(i / nx);
-#pragma unroll
-        for (int a = 0; a < 9; ++a) {
-            const int xs = ex(a) > 0 ? inc1(x, nx) : (ex(a) < 0 ? dec1(x, nx) : x);
-            const int ys = ey(a) > 0 ? inc1(y, ny) : (ey(a) < 0 ? dec1(y, ny) : y);
-            fs[a * n + i] = wt<float>(a) * dev[(size_t)ys * nx + xs];
+            const size_t at = (ey(a) > 0 ? rd : (ey(a) < 0 ? ru : row)) + (ex(a) > 0 ? xl : (ex(a) < 0 ? xr : x));
+            if constexpr (sizeof(T) == sizeof(float)) fs[a * n + at] = wt<float>(a) * d;
+            else fs[a * n + at] = T(wt<double>(a) * r - wt<double>(a) * rho_ref);
         }
     }
 }
