@@ -39,6 +39,7 @@ struct lbm_ctx {
     TilePlan tile;          // tiles of the generic kernel
     WalkPlan walk;          // its walks of tiles, for larger FP32 lattices (sx == 0: separate tiles)
     bool inject_timeout = false;   // the next step's first stage waits give up at once
+    bool automatic = true;         // config is the automatic choice
     // Asynchronous host I/O, set up by the first lbm_init_density_async or
     // lbm_read_moments_async: one copy stream per direction, and device
     // arrays io = [rho0 staging (n)][moment slot 0 (3n)][moment slot 1 (3n)].
@@ -209,8 +210,9 @@ int launch_step(lbm_ctx* c, int cfg, const void* fin, void* fout, long long firs
 int step_once(lbm_ctx* c)
 {
     const long long first_wait = c->inject_timeout ? 0 : kStageWaitPolls;
+    const int cfg = c->inject_timeout && c->config == 0 ? 1 : c->config;   // (a kernel that stages rows)
     c->inject_timeout = false;
-    const int s = launch_step(c, c->config, c->f[c->cur], c->f[c->cur ^ 1], first_wait);
+    const int s = launch_step(c, cfg, c->f[c->cur], c->f[c->cur ^ 1], first_wait);
     if (s != LBM_OK) return s;
     c->cur ^= 1;
     c->steps += 1;
@@ -664,7 +666,14 @@ int lbm_load(lbm_ctx* c, const char* path)
 int lbm_inject_stage_timeout(lbm_ctx* c)
 {
     if (!c) return LBM_E_INVALID;
-    if (c->config < 1) return LBM_E_UNSUPPORTED;   // the generic kernel has no staged copies
+    // The generic kernel has no staged copies.  Where it is the automatic choice of a lattice that 1024-column
+    // strips (or the first configuration's, below that width) would fill, the step of the injection takes strips.
+    if (c->config < 1) {
+        if (!c->automatic || !lbm_strip_supported(&c->p)) return LBM_E_UNSUPPORTED;
+        const long long width = c->p.precision == LBM_FP32_DEV && c->p.nx >= 1024
+                                    ? 1024 : 4LL * lbm_strip_config(c->p.precision, 0).threads;
+        if ((c->p.nx + width - 1) / width * std::max(1, c->p.ny / 16) < sm_count()) return LBM_E_UNSUPPORTED;
+    }
     c->inject_timeout = true;
     return LBM_OK;
 }
@@ -681,6 +690,7 @@ int lbm_set_variant(lbm_ctx* c, int variant)
     if (!c || variant < -1 || variant > 1) return LBM_E_INVALID;
     if (variant == 1 && !lbm_strip_supported(&c->p)) return LBM_E_UNSUPPORTED;
     c->config = variant == -1 ? default_config(c->p) : variant;
+    c->automatic = variant == -1;
     return LBM_OK;
 }
 
@@ -718,6 +728,7 @@ int lbm_set_config(lbm_ctx* c, int config)
 {
     if (!c || config < 0 || config >= n_configs(c->p)) return LBM_E_INVALID;
     c->config = config;
+    c->automatic = false;
     return LBM_OK;
 }
 
@@ -751,6 +762,7 @@ int lbm_autotune(lbm_ctx* c, int trial_steps, int* config, double* ms_per_step)
     cudaEventDestroy(e1);
     if (status != LBM_OK) return status;
     c->config = best;
+    c->automatic = false;
     if (config) *config = best;
     if (ms_per_step) *ms_per_step = best_ms;
     return LBM_OK;

@@ -53,3 +53,27 @@ def test_tile_walks(lbm, nx, ny, coll, forc):
     assert ost == 0 and st["status"] == 0
     assert (np.abs(f.sum(0) - ref.sum(0)) / ref.sum(0)).max() < 2e-5
     assert np.abs(f - ref).max() < 2e-5 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("precision,nx,ny", [("fp64", 1024, 1024), ("fp32", 512, 4096), ("fp32", 1536, 1536)])
+def test_injected_timeout_where_the_generic_kernel_is_the_automatic_choice(lbm, precision, nx, ny):
+    """Generic kernel by default, but strips fill the GPU too, so the step of
+    the injection takes them; a caller's choice of the generic kernel, and a
+    lattice that strips do not fill, refuse it."""
+    p = lbm.make_params(nx, ny, 0.8, 0.9, -0.304, 1.0, "mrt", "guo", precision, **MRT)
+    with lbm.Lattice(p) as lat:
+        assert lat.config == 0
+        lat.init_preset("droplet", 100.0)
+        lat.step(2)
+        lat.inject_stage_timeout()
+        lat.step(1)
+        assert lat.stats()["status"] == lbm.E_TIMEOUT
+        lat.init_preset("droplet", 100.0)
+        lat.step(3)
+        assert lat.stats()["status"] == 0
+        lat.variant = 0
+        with pytest.raises(lbm.LbmError):
+            lat.inject_stage_timeout()
+    with lbm.Lattice(lbm.make_params(64, 64, 0.8, 0.9, -0.304, 1.0, "mrt", "guo", precision, **MRT)) as lat:
+        with pytest.raises(lbm.LbmError):
+            lat.inject_stage_timeout()
