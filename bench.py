@@ -40,12 +40,13 @@ BYTES_PER_NODE = 72          # 9 FP32 deviations read + 9 written
 SEED = 20141217 + 2 * 1000
 
 # DRAM bytes (read + write) per launch of the step kernel measured by ncu on
-# the workload above (mean of three launches: dram__bytes_read.sum +
+# the workload above (one launch: dram__bytes_read.sum +
 # dram__bytes_write.sum), keyed by the sha256 of the kernel sources it was
 # taken from, the kernel configuration id and the lattice side; when any of
 # them changes the entry no longer matches and traffic is null.
 TRAFFIC_CAPTURES: dict = {
-    ("d3cab8f8399c678b", 10, 4096): (604.09e6 + 546.61e6),
+    ("3b8086d784f35703", 10, 4096): (604.08e6 + 548.31e6),
+    ("3b8086d784f35703", 12, 4096): (612.66e6 + 552.19e6),
 }
 # Sources of the block-strip step kernel (its configuration table included).
 KERNEL_SOURCES = ["paper_1412_5170_gb300/csrc/lbm_strip.cuh", "paper_1412_5170_gb300/csrc/lbm_strip_f32.cu",
@@ -717,12 +718,10 @@ def _solution(fn, *a):
 # on one launch of the autotuned kernel
 # (sm__sass_thread_inst_executed_op_{dfma,dadd,dmul}_pred_on.sum / nodes),
 # keyed like TRAFFIC_CAPTURES (sha256 of the kernel sources, configuration
-# id, lattice side); unknown otherwise.  (Counted on the sources before the
-# FP32 density's summation order changed -- an `if constexpr` on float that
-# leaves the FP64 kernel's code as it was.)
+# id, lattice side); unknown otherwise.
 FP64_INST_CAPTURES: dict = {
-    ("d3cab8f8399c678b", 0, 1024): {"dfma": 73662464 / 1048576, "dadd": 87670784 / 1048576,
-                                    "dmul": 40845312 / 1048576},
+    ("3b8086d784f35703", 0, 1024): {"dfma": 65036288 / 1048576, "dadd": 77741056 / 1048576,
+                                    "dmul": 34810368 / 1048576},
 }
 
 
