@@ -288,7 +288,7 @@ k_observe_strip(const T* __restrict__ fin, int nx, int ny, int nchunks, Coef<C> 
     } else if (y1 > y0) {
         strip_init_barriers(sm);
         unsigned G = 0;
-        strip_walk<T, C, NT, NS, true, false, true>(fin, nx, ny, x0, y0, y1, (blockIdx.y & 1) != 0, k, sm, G, bad,
+        strip_walk<T, C, NT, NS, true, true, true>(fin, nx, ny, x0, y0, y1, (blockIdx.y & 1) != 0, k, sm, G, bad,
                                                     row);
     }
     if (!(mode & OBS_REDUCE)) return;
@@ -374,7 +374,10 @@ int launch_walk(const lbm_params* p, const void* f, int mode, double* rho, doubl
 // and strip walk: 64 x 64 37 and 72 us (FP64 50 and 370), 512 x 512 50 and 73
 // (FP64 124 and 358), 1024 x 1024 52 and 74 (FP64 353 and 385), 512 x 4096
 // 108 and 76, 1536 x 1536 112 and 80, 4096 x 4096 301 and 188 (FP64 from
-// 1536 x 1536 on within 1 % of each other).
+// 1536 x 1536 on within 1 % of each other).  Strips of 512 columns, four CTAs
+// of 128 threads an SM, the left halo's psi off the copying warp: with three
+// lattices in turn and snapshots 75.8 us at 1536 x 1536 and 212.2 at
+// 4096 x 4096; 1024 columns take 89.9 and 224.6, 2048 columns 99.8 and 249.6.
 constexpr long long kObsStripNodes = 3 << 19;
 
 int observe_launch(const lbm_params* p, const void* f, int mode, double* rho, double* vx, double* vy, void* vsnap,
@@ -383,7 +386,7 @@ int observe_launch(const lbm_params* p, const void* f, int mode, double* rho, do
     if (p->precision == LBM_FP64)
         return launch_walk<double, double, 2>(p, f, mode, rho, vx, vy, vsnap, parts, ticket, ds, status, nsm, s);
     if (lbm_strip_supported(p) && (long long)p->nx * p->ny >= kObsStripNodes)
-        return launch_strip<float, float, 256, 2, 2>(p, f, mode, rho, vx, vy, vsnap, parts, ticket, ds, status, s);
+        return launch_strip<float, float, 128, 2, 4>(p, f, mode, rho, vx, vy, vsnap, parts, ticket, ds, status, s);
     return launch_walk<float, float, kWalkCtas>(p, f, mode, rho, vx, vy, vsnap, parts, ticket, ds, status, nsm, s);
 }
 
