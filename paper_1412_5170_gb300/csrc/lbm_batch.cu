@@ -114,8 +114,8 @@ k_step_batch(const float* __restrict__ fin, float* __restrict__ fout, const BIns
 // the sweep (2.0 M nodes) 58 and 40.
 template <int COLL, int FORC>
 __global__ void __launch_bounds__(kTileThreads)
-k_step_batch_tiles(const float* __restrict__ fin, float* __restrict__ fout, const BInst* __restrict__ inst,
-                   const BStepTile* __restrict__ tiles, const int* __restrict__ state, unsigned* __restrict__ inst_status)
+k_step_batch_tiles(const float* fin, float* fout, const BInst* inst, const BStepTile* tiles, const int* state,
+                   unsigned* inst_status)
 {
     __shared__ float sp[kTilePsi];
     __shared__ Coef<float> sk;
@@ -137,8 +137,8 @@ k_step_batch_tiles(const float* __restrict__ fin, float* __restrict__ fout, cons
 // chunk its CTA walks down, whatever its height.
 template <int COLL, int FORC>
 __global__ void __launch_bounds__(kWalkThreads, kWalkCtas)
-k_step_batch_walk(const float* __restrict__ fin, float* __restrict__ fout, const BInst* __restrict__ inst,
-                  const BStepTile* __restrict__ tiles, const int* __restrict__ state, unsigned* __restrict__ inst_status)
+k_step_batch_walk(const float* fin, float* fout, const BInst* inst, const BStepTile* tiles, const int* state,
+                  unsigned* inst_status)
 {
     __shared__ WalkPsi<float> sm;
     __shared__ Coef<float> sk;

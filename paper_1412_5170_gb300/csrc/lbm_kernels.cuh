@@ -84,7 +84,12 @@ __device__ __forceinline__ void flag_status(unsigned bad, unsigned* status)
 //
 // Launched as a programmatic dependent of the previous kernel on the stream,
 // as the strip step: it touches memory only after griddepcontrol.wait, and
-// lets the next step's CTAs be scheduled while this one runs.
+// lets the next step's CTAs be scheduled while this one runs.  A kernel that
+// starts so takes no __restrict__ pointers: the qualifier says that nothing
+// else writes the memory while the kernel runs, which allows loads through
+// the read-only cache and ahead of the wait, when the grid before may still
+// be writing it.  The functions called after the wait (step_tile, tile_walk)
+// may use it.
 // ---------------------------------------------------------------------------
 constexpr int GTX = 32, GTY = 8;   // observation tiles
 
@@ -139,8 +144,7 @@ __device__ __forceinline__ void step_tile(const T* __restrict__ fin, T* __restri
 
 template <typename T, typename C, int COLL, int FORC>
 __global__ void __launch_bounds__(kTileThreads)
-k_step_generic(const T* __restrict__ fin, T* __restrict__ fout, int nx, int ny, Coef<C> k,
-               unsigned* __restrict__ status)
+k_step_generic(const T* fin, T* fout, int nx, int ny, Coef<C> k, unsigned* status)
 {
     __shared__ C sp[kTilePsi];
     asm volatile("griddepcontrol.wait;" ::: "memory");

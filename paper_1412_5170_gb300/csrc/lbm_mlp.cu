@@ -153,6 +153,9 @@ enum : int { NET_PREDICT = 0, NET_LOSS = 1, NET_GRAD = 2 };
 
 __host__ __device__ constexpr int pad4(int n) { return (n + 3) & ~3; }
 
+// Start of a kernel launched before its predecessor has finished.  Such a
+// kernel takes no __restrict__ pointers (which would allow loads ahead of the
+// wait and through the read-only cache).
 __device__ __forceinline__ void pdl_wait_and_release()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -256,9 +259,8 @@ __device__ __forceinline__ void dot_cols(float (&acc)[RPT], const float* __restr
 // 5 000 to 9 000 cycles.)
 template <int H, int RPT, int MODE>
 __global__ void __launch_bounds__(256, 1)
-k_net(NetShape sh, const float* __restrict__ image, NetScale sc, const float* __restrict__ X,
-      const float* __restrict__ Y, const int* __restrict__ perm, int n, NetBufs buf, float* __restrict__ out,
-      float* __restrict__ row_loss, int* __restrict__ timeout)
+k_net(NetShape sh, const float* image, NetScale sc, const float* X, const float* Y, const int* perm, int n, NetBufs buf,
+      float* out, float* row_loss, int* timeout)
 {
     constexpr int R = H * RPT, NT = 256;
     extern __shared__ __align__(16) float sm[];
@@ -412,8 +414,7 @@ k_net(NetShape sh, const float* __restrict__ image, NetScale sc, const float* __
 // them.
 template <bool ADAM>
 __global__ void __launch_bounds__(256)
-k_net_grad(NetShape sh, NetBufs buf, int n, float* __restrict__ params, float* __restrict__ image,
-           float* __restrict__ grads, float* __restrict__ m1, float* __restrict__ m2, Adam h)
+k_net_grad(NetShape sh, NetBufs buf, int n, float* params, float* image, float* grads, float* m1, float* m2, Adam h)
 {
     __shared__ float sd[64][TS], sa[64][TS];
     int l = 0, tile = blockIdx.x, ti = 0;

@@ -378,8 +378,7 @@ __device__ __forceinline__ bool strip_walk_step(const T* __restrict__ fin, T* __
 // SM that a CTA of this grid has yet to start on.
 template <typename T, typename C, int COLL, int FORC, int NT, int NS, bool CARRY, int MINB, bool HALO1, bool PSEAM>
 __global__ void __launch_bounds__(NT, MINB)
-k_step_strip(const T* __restrict__ fin, T* __restrict__ fout, int nx, int ny, int nchunks, Coef<C> k,
-             unsigned* __restrict__ status, long long first_wait)
+k_step_strip(const T* fin, T* fout, int nx, int ny, int nchunks, Coef<C> k, unsigned* status, long long first_wait)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -121,8 +121,7 @@ __device__ __forceinline__ void tile_walk(const T* __restrict__ fin, int nx, int
 // One lattice: grid (32-column strips, chunks of `rows` rows).
 template <int COLL, int FORC>
 __global__ void __launch_bounds__(kWalkThreads, kWalkCtas)
-k_step_walk(const float* __restrict__ fin, float* __restrict__ fout, int nx, int ny, int rows, Coef<float> k,
-            unsigned* __restrict__ status)
+k_step_walk(const float* fin, float* fout, int nx, int ny, int rows, Coef<float> k, unsigned* status)
 {
     __shared__ WalkPsi<float> sm;
     asm volatile("griddepcontrol.wait;" ::: "memory");
