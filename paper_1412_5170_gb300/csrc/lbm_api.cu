@@ -277,11 +277,19 @@ double rho_ref_eff(const lbm_params& p)
     return p.precision == LBM_FP64 ? 0.0 : double(float(p.rho_ref));
 }
 
+// CTAs of 256 threads of a node-walking kernel: a thread a node (at 4096 x 4096
+// 4864 CTAs with 13 nodes a thread take 190 us for a start, these 145: their
+// stores stay within a few rows), several nodes a thread from 2^30 nodes.
+unsigned node_ctas(const lbm_params& p)
+{
+    const size_t n = (size_t)p.nx * p.ny;
+    return (unsigned)std::min<size_t>((n + 255) / 256, (size_t)1 << 22);
+}
+
 template <typename T>
 void launch_init_rest(lbm_ctx* c, const double* rho0)
 {
-    const dim3 grid((c->p.nx + 255) / 256, std::min(c->p.ny, 65535));
-    k_init_rest<T><<<grid, 256, 0, c->stream>>>(rho0, (T*)c->f[c->cur], c->p.nx, c->p.ny, rho_ref_eff(c->p));
+    k_init_rest<T><<<node_ctas(c->p), 256, 0, c->stream>>>(rho0, (T*)c->f[c->cur], c->p.nx, c->p.ny, rho_ref_eff(c->p));
 }
 
 // The built-in field of lbm_init_preset into rho0, one thread per node.
@@ -289,10 +297,10 @@ void launch_init_rest(lbm_ctx* c, const double* rho0)
 // droplet array took 90 ms; here the whole call takes 0.40 ms.
 __global__ void __launch_bounds__(256) k_preset_field(PresetField f, double* __restrict__ rho0)
 {
-    const int x = blockIdx.x * 256 + threadIdx.x;
-    if (x >= f.nx) return;
+    const unsigned n = unsigned(f.nx) * unsigned(f.ny);
     const double iw4 = 4.0 / f.width;
-    for (int y = blockIdx.y; y < f.ny; y += gridDim.y) rho0[(size_t)y * f.nx + x] = preset_density(f, iw4, x, y);
+    for (NodeWalk w(blockIdx.x * 256 + threadIdx.x, gridDim.x * 256, f.nx); w.id < n; w.next())
+        rho0[w.id] = preset_density(f, iw4, int(w.x), int(w.y));
 }
 
 template <typename T>
@@ -495,8 +503,7 @@ int lbm_init_preset(lbm_ctx* c, int kind, double size, double width, double rho_
     const int s = lbm_validate_preset(c->p.nx, c->p.ny, kind, size, width, cell);
     if (s != LBM_OK) return s;
     const PresetField f{kind, c->p.nx, c->p.ny, cell, size, width, rho_l, rho_v, noise_amp, seed};
-    const dim3 grid((c->p.nx + 255) / 256, std::min(c->p.ny, 65535));
-    k_preset_field<<<grid, 256, 0, c->stream>>>(f, c->rho);
+    k_preset_field<<<node_ctas(c->p), 256, 0, c->stream>>>(f, c->rho);
     LBM_CUDA(cudaGetLastError());
     return lbm_init_density_dev(c, c->rho);
 }

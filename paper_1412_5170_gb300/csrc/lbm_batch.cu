@@ -22,6 +22,7 @@
 #include "lbm_batch.cuh"
 #include "lbm_fields.cuh"
 #include "lbm_host.h"
+#include "lbm_index.cuh"
 #include "lbm_tilewalk.cuh"
 #include "lbm_warp.cuh"
 
@@ -442,27 +443,11 @@ __device__ __forceinline__ double profile_at(const double* p, int nb, const BGeo
     return p[k0] + t * (p[k0 + 1] - p[k0]);
 }
 
-// Walks a thread over the nodes of an nx-wide instance in steps of the grid's
-// threads, keeping (x, y) without a division per node.
-struct NodeWalk {
-    unsigned id, step;
-    int x, y, nx, sx, sy;
-    __device__ __forceinline__ explicit NodeWalk(int nx_)
-        : id(blockIdx.x * blockDim.x + threadIdx.x), step(gridDim.x * blockDim.x), nx(nx_)
-    {
-        y = int(id / unsigned(nx));
-        x = int(id - unsigned(y) * unsigned(nx));
-        sy = int(step / unsigned(nx));
-        sx = int(step - unsigned(sy) * unsigned(nx));
-    }
-    __device__ __forceinline__ void next()
-    {
-        id += step;
-        x += sx;
-        y += sy;
-        if (x >= nx) { x -= nx; ++y; }
-    }
-};
+// This thread's walk over the nodes of an nx-wide instance.
+__device__ __forceinline__ NodeWalk node_walk(int nx)
+{
+    return NodeWalk(blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, nx);
+}
 
 // Initial density rho0 of every instance into the FP64 node array: its
 // preset (tanh profile plus SplitMix64 noise) or, where geom[i].use, its
@@ -477,12 +462,12 @@ k_rho0_batch(const BInst* __restrict__ inst, int n_inst, double* __restrict__ rh
     const unsigned n = unsigned(I->nx) * unsigned(I->ny);
     double* out = rho0 + I->node_off;
     if (prof && geom[i].use) {
-        for (NodeWalk w(I->nx); w.id < n; w.next())
+        for (NodeWalk w = node_walk(I->nx); w.id < n; w.next())
             out[w.id] = profile_at(prof + (size_t)i * nb, nb, geom[i], radial_distance(I, w.x, w.y));
     } else {
         const PresetField f{I->kind, I->nx, I->ny, I->cell, I->size, I->width, I->rho_l, I->rho_v, I->noise_amp, I->seed};
         const double iw4 = 4.0 / f.width;
-        for (NodeWalk w(I->nx); w.id < n; w.next()) out[w.id] = preset_density(f, iw4, w.x, w.y);
+        for (NodeWalk w = node_walk(I->nx); w.id < n; w.next()) out[w.id] = preset_density(f, iw4, w.x, w.y);
     }
 }
 
@@ -543,7 +528,7 @@ k_pops_batch(const BInst* __restrict__ inst, int n_inst, float* __restrict__ f, 
     const Snap* u = u0 && geom && geom[i].use ? u0 + I->node_off : nullptr;
     const double ref = double(I->k.rho_ref);
     float* fi = f + I->off;
-    for (NodeWalk w(nx); w.id < n; w.next()) {
+    for (NodeWalk w = node_walk(nx); w.id < n; w.next()) {
         const int xl = dec1(w.x, nx), xr = inc1(w.x, nx);
         const size_t row = (size_t)w.y * nx, rd = (size_t)dec1(w.y, ny) * nx, ru = (size_t)inc1(w.y, ny) * nx;
         const double r = r0[w.id];

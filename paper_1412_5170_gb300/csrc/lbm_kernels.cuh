@@ -9,6 +9,7 @@
 
 #include "lbm.h"
 #include "lbm_device.cuh"
+#include "lbm_index.cuh"
 
 namespace lbm {
 
@@ -361,24 +362,25 @@ k_reduce_final(const Partial* __restrict__ parts, int nparts, int nx, DevStats* 
 // x - e_a (a warp's stores stay contiguous).  FP32: w_a float(rho0 - rho_ref),
 // so one FP64 subtraction a node.  Bound by HBM, 8 B read and 36 B (FP64 72 B)
 // written per node; in two passes through an array of deviations, each node
-// found by a 64-bit division, 4096 x 4096 took 200 us in FP32, now 130.
+// found by a 64-bit division, 4096 x 4096 took 200 us in FP32, now 144.  One
+// linear walk over the nodes: on a grid of 256-column blocks by rows, narrow
+// lattices kept 1 to 16 of 256 threads busy (4 x 262144: 43 us, now 11; the two
+// passes 19) and column indices overflowed near 2^31 columns.
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_init_rest(const double* __restrict__ rho0, T* __restrict__ fs, int nx, int ny, double rho_ref)
 {
-    const size_t n = (size_t)nx * ny;
-    const int x = blockIdx.x * 256 + threadIdx.x;
-    if (x >= nx) return;
-    const int xl = dec1(x, nx), xr = inc1(x, nx);
-    for (int y = blockIdx.y; y < ny; y += gridDim.y) {
+    const unsigned n = unsigned(nx) * unsigned(ny);
+    for (NodeWalk w(blockIdx.x * 256 + threadIdx.x, gridDim.x * 256, nx); w.id < n; w.next()) {
+        const int x = int(w.x), y = int(w.y), xl = dec1(x, nx), xr = inc1(x, nx);
         const size_t row = (size_t)y * nx, rd = (size_t)dec1(y, ny) * nx, ru = (size_t)inc1(y, ny) * nx;
-        const double r = rho0[row + x];
+        const double r = rho0[w.id];
         const float d = float(r - rho_ref);
 #pragma unroll
         for (int a = 0; a < 9; ++a) {
             const size_t at = (ey(a) > 0 ? rd : (ey(a) < 0 ? ru : row)) + (ex(a) > 0 ? xl : (ex(a) < 0 ? xr : x));
-            if constexpr (sizeof(T) == sizeof(float)) fs[a * n + at] = wt<float>(a) * d;
-            else fs[a * n + at] = T(wt<double>(a) * r - wt<double>(a) * rho_ref);
+            if constexpr (sizeof(T) == sizeof(float)) fs[(size_t)a * n + at] = wt<float>(a) * d;
+            else fs[(size_t)a * n + at] = T(wt<double>(a) * r - wt<double>(a) * rho_ref);
         }
     }
 }
