@@ -78,7 +78,7 @@ struct Layout {
 Layout layout_of(const lbm_params& p)
 {
     const size_t n = (size_t)p.nx * p.ny;
-    const size_t tiles = (size_t)((p.nx + GTX - 1) / GTX) * ((p.ny + GTY - 1) / GTY);   // at least the observation's CTAs
+    const size_t tiles = (((size_t)p.nx + GTX - 1) / GTX) * (((size_t)p.ny + GTY - 1) / GTY);   // at least the observation's CTAs
     Layout L;
     size_t o = 0;
     L.f0 = o; o = align256(o + 9 * n * tsize(p));

@@ -34,6 +34,9 @@ double bisect(F f, double lo, double hi, int iters = 200)
 
 bool finite_pos(double v) { return std::isfinite(v) && v > 0; }
 
+// a / b rounded up, a and b positive, for any a up to the largest int.
+int ceil_div(int a, int b) { return a / b + (a % b != 0); }
+
 }  // namespace
 
 extern "C" double lbm_tc(void)
@@ -224,9 +227,9 @@ TilePlan plan_tiles(int nx, int ny, bool fp64, int nsm)
     double best_cost = 0;
     for (int w0 : widths)
         for (int h0 : heights) {
-            const int sx = (nx + w0 - 1) / w0, sy = (ny + h0 - 1) / h0;
+            const int sx = ceil_div(nx, w0), sy = ceil_div(ny, h0);
             if (sy > 65535) continue;
-            const int w = (nx + sx - 1) / sx, h = (ny + sy - 1) / sy;   // the largest tile
+            const int w = ceil_div(nx, sx), h = ceil_div(ny, sy);   // the largest tile
             if (w * h > 256 || (w + 2) * (h + 2) > 400) continue;
             const int own = (w * h + 31) / 32, ring = (2 * (w + 2) + 2 * h + 31) / 32;
             if (32 * (own + ring) > 384) continue;
@@ -250,11 +253,11 @@ TilePlan plan_tiles(int nx, int ny, bool fp64, int nsm)
 // 608).
 WalkPlan plan_walk(int nx, int ny, int nsm, int ctas)
 {
-    const int sx = (nx + 31) / 32, tiles = (ny + 7) / 8;
+    const int sx = ceil_div(nx, 32), tiles = ceil_div(ny, 8);
     WalkPlan best{0, 0, 0};
     double best_cost = 0;
     for (int m = 1; m <= tiles && (m <= 512 || best.sx == 0); ++m) {
-        const int sy = (tiles + m - 1) / m;
+        const int sy = ceil_div(tiles, m);
         if (sy > 65535) continue;
         const double f = double(sx) * sy / (double(ctas) * nsm);
         const double cost = (f <= 1 ? 1.1 : f + 0.5 / f) * (m + 0.5);

@@ -315,19 +315,20 @@ k_observe_walk(const T* __restrict__ fin, int nx, int ny, int rows, Coef<C> k, i
     __shared__ WalkPsi<C> sm;
     __shared__ double red[7 * NW], row_sums[2];
     __shared__ unsigned sbad[NW], last;
-    const int x0 = blockIdx.x * kWalkW, y0 = blockIdx.y * rows, y1 = min(y0 + rows, ny), w = min(kWalkW, nx - x0);
+    const RowChunk c = row_chunk(blockIdx.y, rows, ny);
+    const int x0 = blockIdx.x * kWalkW, w = min(kWalkW, nx - x0);
     if (threadIdx.x < 2) row_sums[threadIdx.x] = 0.0;   // (the walk's barriers come before any row's sum)
     ObsNode<C> node{{mode, nx, ny, rho_o, vx_o, vy_o, (mode & OBS_REDUCE) ? ds : nullptr}, vsnap, row_sums, w, {}};
     unsigned bad = 0;
-    tile_walk<T, C>(fin, nx, ny, x0, w, y0, y1, k, sm, bad, node);
+    tile_walk<T, C>(fin, nx, ny, x0, w, c.y0, c.y1, k, sm, bad, node);
     if (!(mode & OBS_REDUCE)) return;
     __syncthreads();
     if (threadIdx.x == 0) {
         node.acc.row_mid = row_sums[0];
         node.acc.row0 = row_sums[1];
     }
-    reduce_and_fold<C, kWalkThreads>(node.acc, bad, double(y1 - y0) * double(w), k, nx, red, sbad, &last, parts, ticket, ds,
-                                     status);
+    reduce_and_fold<C, kWalkThreads>(node.acc, bad, double(c.y1 - c.y0) * double(w), k, nx, red, sbad, &last, parts, ticket,
+                                     ds, status);
 }
 
 template <typename T, typename C, int NT, int NS, int MINB>

@@ -67,7 +67,8 @@ __device__ __forceinline__ void tile_walk(const T* __restrict__ fin, int nx, int
     const int side = r - (w + 2);   // 0 .. 15: row side / 2 of the left (even) or right (odd) column
     const int lx = mine ? lane : (below ? r - 1 : (side & 1 ? w : -1));
     const bool used = mine ? lane < w : (below || side < 2 * kWalkH);
-    const int xs = x0 + lx < 0 ? nx - 1 : (x0 + lx >= nx ? 0 : x0 + lx);   // idle lanes of a ragged strip: any column
+    // (idle lanes of a ragged strip: any column; x0 + lx itself may exceed 2^31 - 1 there)
+    const int xs = lx < -x0 ? nx - 1 : (lx >= nx - x0 ? 0 : x0 + lx);
     const int xm = dec1(xs, nx), xp = inc1(xs, nx);
     // row of this thread's node in a tile of h rows
     auto row_of = [&](int h) { return mine ? wid : (below ? h : side >> 1); };
@@ -112,10 +113,7 @@ __device__ __forceinline__ void tile_walk(const T* __restrict__ fin, int nx, int
         }
         h = hn;
     };
-    for (int y = y0; y < y1; y += 2 * kWalkH) {
-        body(y, 0, gA, gB);
-        if (y + kWalkH < y1) body(y + kWalkH, 1, gB, gA);
-    }
+    walk_tiles<kWalkH>(y0, y1, [&](int y) { body(y, 0, gA, gB); }, [&](int y) { body(y, 1, gB, gA); });
 }
 
 // One lattice: grid (32-column strips, chunks of `rows` rows).
@@ -127,10 +125,10 @@ k_step_walk(const float* fin, float* fout, int nx, int ny, int rows, Coef<float>
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int x0 = blockIdx.x * kWalkW;
-    const int y0 = blockIdx.y * rows;
+    const RowChunk c = row_chunk(blockIdx.y, rows, ny);
     unsigned bad = 0;
     StepNode<float, float, COLL, FORC> node{fout, nx, (size_t)nx * ny};
-    tile_walk<float, float>(fin, nx, ny, x0, min(kWalkW, nx - x0), y0, min(y0 + rows, ny), k, sm, bad, node);
+    tile_walk<float, float>(fin, nx, ny, x0, min(kWalkW, nx - x0), c.y0, c.y1, k, sm, bad, node);
     flag_status(bad, status);
 }
 
