@@ -690,6 +690,15 @@ int batch_sms()
     return nsm;
 }
 
+void* device_alloc(size_t bytes)
+{
+    void* p = nullptr;
+    if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+    cudaGetLastError();   // (reported by the caller)
+    return nullptr;
+}
+void device_free(void* p) { cudaFree(p); }
+
 // Records of the running instances for the tiled step, which a batch takes
 // unless a strip walk was asked for or timed faster: separate tiles below
 // 3 * 2^20 running nodes or for narrow lattices, walks of tiles from there.
@@ -707,10 +716,10 @@ int build_tiles(lbm_batch* b, const int* host_state)
         nodes += (long long)I.nx * I.ny;
         tiles8 += (long long)((I.nx + 31) / 32) * ((I.ny + 7) / 8);
     }
-    b->use_tiles = b->allow_tiles;
+    b->use_tiles = false;   // until the table is in place
     b->tile_walks = nodes >= kBatchWalkNodes && tiles8 * 256 < 2 * nodes;
     b->nstiles = 0;
-    if (!b->use_tiles || nodes == 0) return LBM_OK;
+    if (!b->allow_tiles || nodes == 0) return LBM_OK;
     // separate tiles: two per SM where the batch is that small, 256 nodes at most (smaller ones cost more
     // ring: 146, 163 and 213 us a step at 256, 128 and 64 nodes on 7.5 M nodes).  Walks: chunks of at most
     // 64 rows (25 M nodes: 429 us at 80 rows, 439 at 160, 469 at 320)
@@ -737,16 +746,12 @@ int build_tiles(lbm_batch* b, const int* host_state)
                 t.push_back(BStepTile{I.off, i, I.nx, I.ny, x0, y0, x1 - x0, y1 - y0, 0});
             }
     }
-    if ((int)t.size() > b->stiles_cap) {
-        if (b->stiles) cudaFree(b->stiles);
-        b->stiles = nullptr;
-        b->stiles_cap = 0;
-        B_CUDA(cudaMalloc(&b->stiles, sizeof(BStepTile) * t.size()));
-        b->stiles_cap = (int)t.size();
-    }
+    // no room for the table: the batch steps on the strip walks, whose items are in place
+    if (!table_reserve(b->stiles, b->stiles_cap, t.size(), device_alloc, device_free)) return LBM_OK;
     B_CUDA(cudaMemcpyAsync(b->stiles, t.data(), sizeof(BStepTile) * t.size(), cudaMemcpyHostToDevice, b->stream));
     B_CUDA(cudaStreamSynchronize(b->stream));
     b->nstiles = (int)t.size();
+    b->use_tiles = true;
     return LBM_OK;
 }
 
@@ -771,10 +776,10 @@ int build_items(lbm_batch* b, const int* host_state)
     const long long target = 16LL * nsm;
     const int rows = (int)std::max<long long>(std::min<long long>(b->rows, strip_rows / target), std::min(4, b->rows));
     std::vector<BItem> it;
-    b->items_for = 0;
+    int running = 0;
     for (int i = 0; i < b->n; ++i) {
         if (host_state && host_state[i] != B_RUNNING) continue;
-        b->items_for += 1;
+        running += 1;
         const BInst& I = b->hinst[i];
         const int nstrips = (I.nx + b->cols - 1) / b->cols;
         const int nch = std::max(1, (I.ny + rows / 2) / rows);
@@ -786,11 +791,11 @@ int build_items(lbm_batch* b, const int* host_state)
     }
     // longest items first, so the walkers taking them from the queue finish evenly
     std::stable_sort(it.begin(), it.end(), [](const BItem& a, const BItem& c) { return (a.y1 - a.y0) > (c.y1 - c.y0); });
-    if ((int)it.size() > b->items_cap) {
-        if (b->items) cudaFree(b->items);
-        b->items_cap = std::max<int>(it.size(), 1);
-        B_CUDA(cudaMalloc(&b->items, sizeof(BItem) * b->items_cap));
+    if (!table_reserve(b->items, b->items_cap, std::max<size_t>(it.size(), 1), device_alloc, device_free)) {
+        std::fprintf(stderr, "liblbm (batch): no memory for %zu work items\n", it.size());
+        return LBM_E_CUDA;   // the batch keeps its items
     }
+    b->items_for = running;
     b->nitems = (int)it.size();
     if (b->nitems)
         B_CUDA(cudaMemcpyAsync(b->items, it.data(), sizeof(BItem) * b->nitems, cudaMemcpyHostToDevice, b->stream));
@@ -1289,12 +1294,22 @@ int lbm_batch_set_tuning(lbm_batch* b, int columns, int stages, int rows_per_ite
     } else if (!carry || !((columns == 256 && stages == 3) || (columns == 512 && (stages == 2 || stages == 3)))) {
         return LBM_E_INVALID;
     }
+    const int old[4] = {b->cols, b->ns, b->carry, b->rows};
+    const bool tiles = b->allow_tiles;
     b->cols = columns;
     b->ns = stages;
     b->carry = carry ? 1 : 0;
     b->rows = rows_per_item;
     b->allow_tiles = false;
-    return build_items(b, b->h_state);
+    const int s = build_items(b, b->h_state);
+    if (s != LBM_OK) {   // the items are still those of the old tuning
+        b->cols = old[0];
+        b->ns = old[1];
+        b->carry = old[2];
+        b->rows = old[3];
+        b->allow_tiles = tiles;
+    }
+    return s;
 }
 
 int lbm_batch_autotune(lbm_batch* b, int trial_steps, int* columns, int* stages, int* rows_per_item, int* carry,

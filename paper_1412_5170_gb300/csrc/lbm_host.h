@@ -31,6 +31,21 @@ TilePlan plan_tiles(int nx, int ny, bool fp64, int nsm);
 struct WalkPlan { int sx, sy, rows; };
 WalkPlan plan_walk(int nx, int ny, int nsm, int ctas);
 
+// Room for n records in a device table of cap: the larger buffer is allocated
+// before the old one is given back, so that a failed allocation (alloc returns
+// null; false) leaves the table as it was.
+template <typename T, class Alloc, class Free>
+bool table_reserve(T*& table, int& cap, size_t n, Alloc alloc, Free release)
+{
+    if (n <= (size_t)cap) return true;
+    void* const p = alloc(n * sizeof(T));
+    if (!p) return false;
+    if (table) release(table);
+    table = static_cast<T*>(p);
+    cap = (int)n;
+    return true;
+}
+
 // Polls of a bounded stage wait (mbarrier try_wait) before the staged kernels
 // declare a row copy stuck, flag a timeout, drain and return.
 constexpr long long kStageWaitPolls = 1ll << 26;
