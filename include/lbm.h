@@ -255,8 +255,10 @@ int lbm_load(lbm_ctx *ctx, const char *path);
  * LBM_E_TIMEOUT; re-initialise the state (lbm_init_*, lbm_load,
  * lbm_write_populations) to go on.  LBM_E_UNSUPPORTED if the context runs
  * the generic kernel (configuration 0), which stages nothing, unless that is
- * the automatic choice of a lattice whose strips give every SM a CTA: the
- * step then takes the strip kernel. */
+ * the automatic choice of a lattice whose strips give every SM a CTA: that
+ * one step then takes the strip kernel.  Choosing the generic kernel between
+ * the injection and the step (lbm_set_variant, lbm_set_config) drops the
+ * injection. */
 int lbm_inject_stage_timeout(lbm_ctx *ctx);
 
 /* Kernel variant in use: 0 = generic tiled kernel (any nx), 1 = pipelined

@@ -210,7 +210,8 @@ int launch_step(lbm_ctx* c, int cfg, const void* fin, void* fout, long long firs
 int step_once(lbm_ctx* c)
 {
     const long long first_wait = c->inject_timeout ? 0 : kStageWaitPolls;
-    const int cfg = c->inject_timeout && c->config == 0 ? 1 : c->config;   // (a kernel that stages rows)
+    // the step of an injection takes a kernel that stages rows, unless the caller has chosen another since
+    const int cfg = c->inject_timeout && c->config == 0 && c->automatic ? 1 : c->config;
     c->inject_timeout = false;
     const int s = launch_step(c, cfg, c->f[c->cur], c->f[c->cur ^ 1], first_wait);
     if (s != LBM_OK) return s;
