@@ -299,7 +299,7 @@ void launch_init_rest(lbm_ctx* c, const double* rho0)
 __global__ void __launch_bounds__(256) k_preset_field(PresetField f, double* __restrict__ rho0)
 {
     const unsigned n = unsigned(f.nx) * unsigned(f.ny);
-    const double iw4 = 4.0 / f.width;
+    const double iw4 = preset_inv_width4(f.width);
     for (NodeWalk w(blockIdx.x * 256 + threadIdx.x, gridDim.x * 256, f.nx); w.id < n; w.next())
         rho0[w.id] = preset_density(f, iw4, int(w.x), int(w.y));
 }

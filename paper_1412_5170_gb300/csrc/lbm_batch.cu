@@ -466,7 +466,7 @@ k_rho0_batch(const BInst* __restrict__ inst, int n_inst, double* __restrict__ rh
             out[w.id] = profile_at(prof + (size_t)i * nb, nb, geom[i], radial_distance(I, w.x, w.y));
     } else {
         const PresetField f{I->kind, I->nx, I->ny, I->cell, I->size, I->width, I->rho_l, I->rho_v, I->noise_amp, I->seed};
-        const double iw4 = 4.0 / f.width;
+        const double iw4 = preset_inv_width4(f.width);
         for (NodeWalk w = node_walk(I->nx); w.id < n; w.next()) out[w.id] = preset_density(f, iw4, w.x, w.y);
     }
 }

@@ -23,7 +23,11 @@ __device__ __forceinline__ unsigned long long splitmix64_dev(unsigned long long 
     return z ^ (z >> 31);
 }
 
-// rho0 of node (x, y) (inv_width4 = 4 / width): rho_v + (rho_l - rho_v) in + noise with
+// 4 / width, held finite: below 2e-308 the quotient would be infinite, and a
+// node on the interface (distance 0) 0 * inf instead of halfway.
+__device__ __forceinline__ double preset_inv_width4(double width) { return fmin(4.0 / width, 1.7976931348623157e308); }
+
+// rho0 of node (x, y) (inv_width4 = preset_inv_width4(width)): rho_v + (rho_l - rho_v) in + noise with
 // in = (1 - tanh(2 d / width))/2 and d the signed distance to the liquid (a
 // bubble swaps the phases).
 //
