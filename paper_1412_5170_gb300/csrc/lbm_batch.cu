@@ -162,26 +162,6 @@ constexpr size_t batch_smem() { return batch_coef_off<NS>() + kBatchWarps * size
 
 enum : int { BO_RHO = 1, BO_SNAP = 2, BO_ALL = 4 };
 
-// Sum of floats held as an unevaluated pair (s, e): Knuth's TwoSum keeps each
-// addition's rounding in e, so the pair is good to about 2^-45 without the
-// FP64 pipe.
-struct FPair { float s, e; };
-__device__ __forceinline__ FPair pair_add(FPair a, FPair b)
-{
-    const float t = a.s + b.s, bp = t - a.s;
-    return FPair{t, (a.e + b.e) + ((a.s - (t - bp)) + (b.s - bp))};
-}
-// Its value in FP64 (an infinite or NaN sum leaves no rounding to add).
-__device__ __forceinline__ double pair_value(FPair p) { return isfinite(p.e) ? double(p.s) + double(p.e) : double(p.s); }
-__device__ __forceinline__ FPair warp_pair_sum(float v)
-{
-    FPair p{v, 0.f};
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        p = pair_add(p, FPair{__shfl_xor_sync(0xffffffffu, p.s, o), __shfl_xor_sync(0xffffffffu, p.e, o)});
-    return p;
-}
-
 // Observables per 32 x 8 tile of every running instance (every instance with
 // BO_ALL): rho and v = u + F/(2 rho); with BO_SNAP the changes against the
 // snapshot (vx, vy, rho) of the previous check, which is then replaced; with
@@ -189,11 +169,14 @@ __device__ __forceinline__ FPair warp_pair_sum(float v)
 //
 // Eight warps take the tile's rows and three the ring of nodes around it, so
 // that every node is pulled and its psi evaluated once, from one round of
-// loads.  All per-node and per-warp work is FP32: maxima are exact in any
-// precision, the sums of drho are float pairs, and one thread per tile turns
-// seven numbers into FP64.  (With FP64 shuffle sums and the pull repeated
-// after the psi pass lbm_batch_observe took 1.57 ms on the 25 M nodes of 256
-// sweep instances; now 0.71, of which the populations' way from HBM is 0.13.)
+// loads.  All per-node work is FP32, and maxima are exact in any precision.
+// The sums of drho (mass and probe rows) are FP64: the tile's deviations go to
+// shared memory, one warp adds each column down and then across, 13 FP64
+// additions a tile for the mass where shuffle sums in every row's warp took
+// 40.  (With those and the pull repeated after the psi pass lbm_batch_observe
+// took 1.57 ms on the 25 M nodes of 256 sweep instances, with pairs of floats
+// in place of FP64 sums 0.71, and so no more; the populations' way from HBM is
+// 0.13 of it.)
 constexpr int kObsThreads = 32 * (GTY + 3);
 __global__ void __launch_bounds__(kObsThreads)
 k_observe_batch(const float* __restrict__ f, const BInst* __restrict__ inst, const BTile* __restrict__ tiles,
@@ -201,7 +184,7 @@ k_observe_batch(const float* __restrict__ f, const BInst* __restrict__ inst, con
                 BPart* __restrict__ parts, BObs* __restrict__ obs, int mode)
 {
     __shared__ float sp[(GTY + 2) * (GTX + 2)];
-    __shared__ float red[11][GTY];
+    __shared__ float red[5][GTY], sd[GTY][GTX];
     __shared__ unsigned sbad;
     const BTile tl = tiles[blockIdx.x];
     if (!(mode & BO_ALL) && state[tl.inst] != B_RUNNING) return;   // uniform over the block
@@ -276,37 +259,34 @@ k_observe_batch(const float* __restrict__ f, const BInst* __restrict__ inst, con
         ndmin = -drho;
     }
     if (wid < GTY) {   // a warp is one tile row
-        const FPair m = warp_pair_sum(drho);
-        const bool mid_row = y == ny / 2, row_0 = y == 0;
-        const float r[9] = {m.s, m.e, mid_row ? m.s : 0.f, mid_row ? m.e : 0.f, row_0 ? m.s : 0.f, row_0 ? m.e : 0.f,
-                            warp_max(mv), warp_max(dv), warp_max(dr)};
-        const float r9 = warp_max(dmax), r10 = warp_max(ndmin);
+        sd[wid][lx] = drho;   // (0 beyond the tile)
+        const float r[5] = {warp_max(mv), warp_max(dv), warp_max(dr), warp_max(dmax), warp_max(ndmin)};
         if ((t & 31) == 0) {
 #pragma unroll
-            for (int j = 0; j < 9; ++j) red[j][wid] = r[j];
-            red[9][wid] = r9;
-            red[10][wid] = r10;
+            for (int j = 0; j < 5; ++j) red[j][wid] = r[j];
         }
     }
     const unsigned wb = __reduce_or_sync(0xffffffffu, bad);
     if ((t & 31) == 0 && wb) atomicOr(&sbad, wb);
     __syncthreads();
+    if (wid > 0) return;
+    double m = 0.0;
+#pragma unroll
+    for (int i = 0; i < GTY; ++i) m += double(sd[i][t]);
+    m = warp_sum(m);
+    const bool has_mid = ny / 2 >= y0 && ny / 2 < y0 + h;   // uniform over the CTA
+    const double mid = has_mid ? warp_sum(double(sd[ny / 2 - y0][t])) : 0.0;
+    const double r0 = y0 == 0 ? warp_sum(double(sd[0][t])) : 0.0;
     if (t == 0) {
-        FPair m{0.f, 0.f}, mid{0.f, 0.f}, r0{0.f, 0.f};
         float mx[5] = {0.f, 0.f, 0.f, -1e30f, -1e30f};
-        for (int i = 0; i < h; ++i) {
-            m = pair_add(m, FPair{red[0][i], red[1][i]});
-            mid = pair_add(mid, FPair{red[2][i], red[3][i]});
-            r0 = pair_add(r0, FPair{red[4][i], red[5][i]});
-            for (int j = 0; j < 5; ++j) mx[j] = fmaxf(mx[j], red[6 + j][i]);
-        }
+        for (int i = 0; i < h; ++i)
+            for (int j = 0; j < 5; ++j) mx[j] = fmaxf(mx[j], red[j][i]);
         // sum of rho = nodes rho_ref + sum of drho
         const double ref = double(k.rho_ref);
-        const bool has_mid = ny / 2 >= y0 && ny / 2 < y0 + h;
         BPart p;
-        p.sum[0] = double(w * h) * ref + pair_value(m);
-        p.sum[1] = has_mid ? double(w) * ref + pair_value(mid) : 0.0;
-        p.sum[2] = y0 == 0 ? double(w) * ref + pair_value(r0) : 0.0;
+        p.sum[0] = double(w * h) * ref + m;
+        p.sum[1] = has_mid ? double(w) * ref + mid : 0.0;
+        p.sum[2] = y0 == 0 ? double(w) * ref + r0 : 0.0;
         p.mx[0] = double(mx[0]);
         p.mx[1] = double(mx[1]);
         p.mx[2] = double(mx[2]);
