@@ -22,18 +22,20 @@ namespace lbm {
 namespace {
 
 // Running reductions of one thread, and the probe rows' sums.  The mass is
-// N rho_ref plus the sum of the deviations drho: in FP64 for an FP64 lattice;
-// for FP32 deviations a float pair (sum, error) kept by Knuth's TwoSum, which
-// carries every addition's rounding exactly into the error term (six FP32
+// N rho_ref plus the sum of the deviations drho, in FP64.  PAIR (strips of FP32
+// deviations): a float pair (sum, error) kept by Knuth's TwoSum, which
+// carries every addition's rounding into the error term (six FP32
 // additions a node instead of a conversion and an addition on this GPU's
-// narrow FP64 pipe), converted to FP64 once per thread.  The maxima are taken
+// narrow FP64 pipe), converted to FP64 once per thread.  The walks of tiles,
+// which also serve widths whose sums were never pairs, hide one FP64 addition
+// a node behind its other 400 instructions.  The maxima are taken
 // on |v|^2 and |v - v_snap|^2 in the compute type (exact) and rooted once per
 // CTA.
-template <typename C>
+template <typename C, bool PAIR>
 struct ObsAcc {
     double dmass = 0.0, row_mid = 0.0, row0 = 0.0;
     C mv2 = C(0), mdv2 = C(0), dmax = -obs_huge<C>(), ndmin = -obs_huge<C>();
-    float ms = 0.f, me = 0.f;   // FP32: running sum of drho and its accumulated rounding
+    float ms = 0.f, me = 0.f;   // PAIR: running sum of drho and its accumulated rounding
 
     __device__ __forceinline__ void node(C d, C vx, C vy)
     {
@@ -41,7 +43,7 @@ struct ObsAcc {
         mv2 = (s2 > mv2 || s2 != s2) ? s2 : mv2;      // NaN wins (reported as huge)
         dmax = d > dmax ? d : dmax;
         ndmin = -d > ndmin ? -d : ndmin;
-        if constexpr (sizeof(C) == sizeof(float)) {
+        if constexpr (PAIR) {
             const float t = ms + d;
             const float bp = t - ms;
             me += (ms - (t - bp)) + (d - bp);
@@ -69,7 +71,7 @@ template <typename T, typename C>
 struct ObsRow {
     ObsOut to;
     VSnap<C>* __restrict__ vsnap;
-    ObsAcc<C> acc;
+    ObsAcc<C, sizeof(C) == sizeof(float)> acc;
     __device__ __forceinline__ void operator()(int y, int x, bool active, C (&gc)[9][4], const C (&rm)[6],
                                                const C (&r0)[6], const C (&rp)[6], const Coef<C>& k,
                                                unsigned& bad)
@@ -129,7 +131,7 @@ struct ObsNode {
     VSnap<C>* __restrict__ vsnap;
     double* __restrict__ rows;   // shared: sums of rho over the strip's part of rows ny/2 and 0
     int w;                       // the strip's width: lanes 0 .. w - 1 hold its columns
-    ObsAcc<C> acc;
+    ObsAcc<C, false> acc;
 
     __device__ __forceinline__ void operator()(int y, int x, C (&g)[9], const Stencil<C>& q, const Coef<C>& k,
                                                unsigned& bad)
@@ -179,15 +181,15 @@ __device__ __forceinline__ double warp_max_root(C v2)
 // The CTA's partial from its threads' reductions (warp shuffles, then the
 // warps in order), and in the last CTA to get here the fold of all partials.
 // red [7 NW], sbad [NW] and last are shared memory.
-template <typename C, int NT>
-__device__ __forceinline__ void reduce_and_fold(ObsAcc<C>& acc, unsigned bad, double cta_nodes, const Coef<C>& k, int nx,
+template <typename C, int NT, bool PAIR>
+__device__ __forceinline__ void reduce_and_fold(ObsAcc<C, PAIR>& acc, unsigned bad, double cta_nodes, const Coef<C>& k, int nx,
                                                 double* red, unsigned* sbad, unsigned* last,
                                                 Partial* __restrict__ parts, unsigned* __restrict__ ticket,
                                                 DevStats* __restrict__ ds, const unsigned* __restrict__ status)
 {
     constexpr int NW = NT / 32;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if constexpr (sizeof(C) == sizeof(float)) acc.dmass = double(acc.ms) + double(acc.me);
+    if constexpr (PAIR) acc.dmass = double(acc.ms) + double(acc.me);
     double v[7] = {warp_sum(acc.dmass), warp_sum(acc.row_mid), warp_sum(acc.row0), warp_max_root(acc.mv2),
                    warp_max_root(acc.mdv2), 0.0, 0.0};
     const C wdmax = warp_max(acc.dmax), wndmin = warp_max(acc.ndmin);
