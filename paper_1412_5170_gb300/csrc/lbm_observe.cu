@@ -12,6 +12,7 @@
 // DevStats record in the same launch: the result is the same bit for bit
 // from run to run.
 #include <algorithm>
+#include <cstddef>
 
 #include "lbm.h"
 #include "lbm_host.h"
@@ -129,8 +130,6 @@ template <typename C>
 struct ObsNode {
     ObsOut to;
     VSnap<C>* __restrict__ vsnap;
-    double* __restrict__ rows;   // shared: sums of rho over the strip's part of rows ny/2 and 0
-    int w;                       // the strip's width: lanes 0 .. w - 1 hold its columns
     ObsAcc<C, false> acc;
 
     __device__ __forceinline__ void operator()(int y, int x, C (&g)[9], const Stencil<C>& q, const Coef<C>& k,
@@ -148,17 +147,10 @@ struct ObsNode {
         const bool mid = y == to.ny / 2;
         if (mid || y == 0 || (mode & OBS_FIELDS)) {   // (uniform over the warp)
             const double rho = double(k.rho_ref) + double(d);
-            if (mid || y == 0) {
-                const unsigned lanes = w == 32 ? 0xffffffffu : (1u << w) - 1u;
-                double s = 0.0;
-                for (int i = 0; i < w; ++i) s += __shfl_sync(lanes, rho, i);
-                if ((threadIdx.x & 31) == 0) {
-                    if (mid) rows[0] = s;
-                    if (y == 0) rows[1] = s;
-                }
-                if (to.ds && mid && x == to.nx / 2) to.ds->rho_center = rho;
-                if (to.ds && y == 0 && x == 0) to.ds->rho_corner = rho;
-            }
+            if (mid) acc.row_mid += rho;
+            if (y == 0) acc.row0 += rho;
+            if (to.ds && mid && x == to.nx / 2) to.ds->rho_center = rho;
+            if (to.ds && y == 0 && x == 0) to.ds->rho_corner = rho;
             if (mode & OBS_FIELDS) {
                 to.rho_o[o] = rho;
                 to.vx_o[o] = double(vx);
@@ -170,16 +162,34 @@ struct ObsNode {
     }
 };
 
-// max over a warp of a squared magnitude, then its root (NaN -> huge)
-template <typename C>
-__device__ __forceinline__ double warp_max_root(C v2)
+// Quantities of a partial in the order of its fields: sums of the mass and of
+// rows ny/2 and 0, maxima of |v|, |v - v_snap|, rho and -rho.
+constexpr int kObsQ = 7, kObsSums = 3;
+static_assert(offsetof(Partial, status) == kObsQ * sizeof(double), "a partial starts with its quantities");
+
+// Quantity `lane` over the warps' values in red, in the warps' order.
+template <int NW>
+__device__ __forceinline__ double fold_warps(const double* red, int lane, double first)
 {
-    const C w = warp_max(v2 != v2 ? obs_huge<C>() : v2);
-    return double(sqrt(w));
+    double x[NW];
+#pragma unroll
+    for (int w = 0; w < NW; ++w) x[w] = red[min(lane, kObsQ - 1) * NW + w];
+    double r = first, m = -1e300;
+    if (lane < kObsSums) {
+#pragma unroll
+        for (int w = 0; w < NW; ++w) r += x[w];
+        return r;
+    }
+#pragma unroll
+    for (int w = 0; w < NW; ++w) m = fmax(m, x[w]);
+    return m;
 }
 
 // The CTA's partial from its threads' reductions (warp shuffles, then the
 // warps in order), and in the last CTA to get here the fold of all partials.
+// One lane of the first warp takes each quantity, so that the serial chain is
+// one FP64 operation a warp and not seven: FP64 operations take 64 cycles
+// here, and a CTA's whole reduction is as long as several rows of its walk.
 // red [7 NW], sbad [NW] and last are shared memory.
 template <typename C, int NT, bool PAIR>
 __device__ __forceinline__ void reduce_and_fold(ObsAcc<C, PAIR>& acc, unsigned bad, double cta_nodes, const Coef<C>& k, int nx,
@@ -190,87 +200,82 @@ __device__ __forceinline__ void reduce_and_fold(ObsAcc<C, PAIR>& acc, unsigned b
     constexpr int NW = NT / 32;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if constexpr (PAIR) acc.dmass = double(acc.ms) + double(acc.me);
-    double v[7] = {warp_sum(acc.dmass), warp_sum(acc.row_mid), warp_sum(acc.row0), warp_max_root(acc.mv2),
-                   warp_max_root(acc.mdv2), 0.0, 0.0};
-    const C wdmax = warp_max(acc.dmax), wndmin = warp_max(acc.ndmin);
-    v[5] = double(k.rho_ref) + double(wdmax);
-    v[6] = -(double(k.rho_ref) + double(-wndmin));
+    // (few warps hold part of a probe row)
+    if (__any_sync(0xffffffffu, acc.row_mid != 0.0)) acc.row_mid = warp_sum(acc.row_mid);
+    if (__any_sync(0xffffffffu, acc.row0 != 0.0)) acc.row0 = warp_sum(acc.row0);
+    const double v[kObsQ] = {warp_sum(acc.dmass), acc.row_mid, acc.row0,
+                             double(warp_max(acc.mv2 != acc.mv2 ? obs_huge<C>() : acc.mv2)),      // |v|^2 (NaN -> huge)
+                             double(warp_max(acc.mdv2 != acc.mdv2 ? obs_huge<C>() : acc.mdv2)),
+                             double(warp_max(acc.dmax)), double(warp_max(acc.ndmin))};
     const unsigned wbad = __reduce_or_sync(0xffffffffu, bad);
     if (lane == 0) {
 #pragma unroll
-        for (int j = 0; j < 7; ++j) red[j * NW + wid] = v[j];
+        for (int j = 0; j < kObsQ; ++j) red[j * NW + wid] = v[j];
         sbad[wid] = wbad;
     }
     __syncthreads();
     const unsigned nparts = gridDim.x * gridDim.y;
-    if (threadIdx.x == 0) {
-        Partial p;
-        p.mass = p.row_mid = p.row0 = 0;
-        p.max_v = p.max_dv = p.rho_max = p.neg_rho_min = -1e300;
-        p.status = 0;
-        p.mass = cta_nodes * double(k.rho_ref);
-        for (int w = 0; w < NW; ++w) {
-            p.mass += red[0 * NW + w]; p.row_mid += red[1 * NW + w]; p.row0 += red[2 * NW + w];
-            p.max_v = fmax(p.max_v, red[3 * NW + w]); p.max_dv = fmax(p.max_dv, red[4 * NW + w]);
-            p.rho_max = fmax(p.rho_max, red[5 * NW + w]); p.neg_rho_min = fmax(p.neg_rho_min, red[6 * NW + w]);
-            p.status |= sbad[w];
-        }
-        p.pad = 0;
-        parts[blockIdx.y * gridDim.x + blockIdx.x] = p;
+    if (wid == 0) {
+        const double ref = double(k.rho_ref);
+        double r = fold_warps<NW>(red, lane, lane == 0 ? cta_nodes * ref : 0.0);
+        const unsigned pb = __reduce_or_sync(0xffffffffu, lane < NW ? sbad[lane] : 0u);
+        // roots and densities of the maxima: both are monotone, so of the CTA's as of each warp's
+        if (lane == 3 || lane == 4) r = double(sqrt(C(r)));
+        else if (lane == 5) r = ref + r;
+        else if (lane == 6) r = -(ref - r);
+        Partial* p = parts + (blockIdx.y * gridDim.x + blockIdx.x);
+        if (lane < kObsQ) reinterpret_cast<double*>(p)[lane] = r;
+        else if (lane == kObsQ) p->status = pb;
         __threadfence();
-        *last = atomicAdd(ticket, 1u) == nparts - 1;
+        __syncwarp();
+        if (lane == 0) *last = atomicAdd(ticket, 1u) == nparts - 1;
     }
     __syncthreads();
     if (!*last) return;
 
-    // The last CTA: every partial is written and fenced; fold them in a fixed
-    // order (thread t takes t, t + NT, ...; then the warps; then thread 0).
+    // The last CTA: every partial is written and fenced.  A warp folds each
+    // quantity in a fixed order (lane l takes partials l, l + 32, ..., then
+    // shuffles), so the three sums run on FP64 pipes of their own.
     __threadfence();
-    double a[7] = {0, 0, 0, -1e300, -1e300, -1e300, -1e300};
-    unsigned b = 0;
-    for (unsigned i = threadIdx.x; i < nparts; i += NT) {
-        const Partial* q = parts + i;
-        a[0] += __ldcg(&q->mass); a[1] += __ldcg(&q->row_mid); a[2] += __ldcg(&q->row0);
-        a[3] = fmax(a[3], __ldcg(&q->max_v)); a[4] = fmax(a[4], __ldcg(&q->max_dv));
-        a[5] = fmax(a[5], __ldcg(&q->rho_max)); a[6] = fmax(a[6], __ldcg(&q->neg_rho_min));
-        b |= __ldcg(&q->status);
-    }
-#pragma unroll
-    for (int j = 0; j < 3; ++j) a[j] = warp_sum(a[j]);
-#pragma unroll
-    for (int j = 3; j < 7; ++j) a[j] = warp_max(a[j]);
-    b = __reduce_or_sync(0xffffffffu, b);
-    __syncthreads();
-    if (lane == 0) {
-#pragma unroll
-        for (int j = 0; j < 7; ++j) red[j * NW + wid] = a[j];
-        sbad[wid] = b;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double f[7] = {0, 0, 0, -1e300, -1e300, -1e300, -1e300};
-        unsigned fb = status ? *status : 0u;
-        for (int w = 0; w < NW; ++w) {
-            for (int j = 0; j < 3; ++j) f[j] += red[j * NW + w];
-            for (int j = 3; j < 7; ++j) f[j] = fmax(f[j], red[j * NW + w]);
-            fb |= sbad[w];
+    for (int q = wid; q <= kObsQ; q += NW) {
+        if (q == kObsQ) {   // the status words
+            unsigned b = 0;
+            for (unsigned i = lane; i < nparts; i += 32) b |= __ldcg(&parts[i].status);
+            b = __reduce_or_sync(0xffffffffu, b);
+            if (lane == 0) ds->status = b | (status ? *status : 0u);
+            continue;
         }
-        ds->mass = f[0];
-        ds->rho_row_mid = f[1] / nx;
-        ds->rho_row0 = f[2] / nx;
-        ds->max_v = f[3];
-        ds->max_dv = f[4];
-        ds->rho_max = f[5];
-        ds->rho_min = -f[6];
-        ds->status = fb;
-        *ticket = 0;   // ready for the next launch
+        const double* x = reinterpret_cast<const double*>(parts) + q;
+        constexpr size_t stride = sizeof(Partial) / sizeof(double);
+        double r = q < kObsSums ? 0.0 : -1e300;
+        if (q < kObsSums) {
+#pragma unroll 8
+            for (unsigned i = lane; i < nparts; i += 32) r += __ldcg(x + i * stride);
+            r = warp_sum(r);
+        } else {
+#pragma unroll 8
+            for (unsigned i = lane; i < nparts; i += 32) r = fmax(r, __ldcg(x + i * stride));
+            r = warp_max(r);
+        }
+        if (lane == 0) {
+            switch (q) {
+            case 0: ds->mass = r; break;
+            case 1: ds->rho_row_mid = r / nx; break;
+            case 2: ds->rho_row0 = r / nx; break;
+            case 3: ds->max_v = r; break;
+            case 4: ds->max_dv = r; break;
+            case 5: ds->rho_max = r; break;
+            case 6: ds->rho_min = -r; break;
+            }
+        }
     }
+    if (threadIdx.x == 0) *ticket = 0;   // ready for the next launch
 }
 
 // One CTA per (strip, row chunk), as the step kernel.  Every CTA reaches the
 // reduction, whatever happened to its walk (a misaligned buffer, an empty
 // chunk, a stage wait that gave up), so the ticket always completes.
-template <typename T, typename C, int NT, int NS, int MINB>
+template <typename T, typename C, int NT, int NS, int MINB, bool HALO1>
 __global__ void __launch_bounds__(NT, MINB)
 k_observe_strip(const T* __restrict__ fin, int nx, int ny, int nchunks, Coef<C> k, int mode,
                 double* __restrict__ rho_o, double* __restrict__ vx_o, double* __restrict__ vy_o,
@@ -290,7 +295,7 @@ k_observe_strip(const T* __restrict__ fin, int nx, int ny, int nchunks, Coef<C> 
     } else if (y1 > y0) {
         strip_init_barriers(sm);
         unsigned G = 0;
-        strip_walk<T, C, NT, NS, true, true, true>(fin, nx, ny, x0, y0, y1, (blockIdx.y & 1) != 0, k, sm, G, bad,
+        strip_walk<T, C, NT, NS, true, HALO1, true>(fin, nx, ny, x0, y0, y1, (blockIdx.y & 1) != 0, k, sm, G, bad,
                                                     row);
     }
     if (!(mode & OBS_REDUCE)) return;
@@ -305,41 +310,45 @@ k_observe_strip(const T* __restrict__ fin, int nx, int ny, int nchunks, Coef<C> 
     reduce_and_fold<C, NT>(row.acc, bad, cta_nodes, k, nx, red, sbad, sbad + NW, parts, ticket, ds, status);
 }
 
-// The same with the walk of tiles: one CTA per (32-column strip, chunk of `rows` rows).
+// The same with the walk of tiles: `items` pieces of the lattice, each a
+// 32-column strip's chunk of `rows` rows, shared out over the grid's CTAs, so
+// that a CTA reduces once whatever the lattice's shape.  (With a CTA a piece,
+// wide flat lattices were mostly reductions: lbm_stats at 65536 x 16 took 105
+// us, now 51; 4096 x 256 100, now 51.)  Pieces of more than 64 rows are worth
+// a CTA each, which evens out the last wave: 2047 x 2049 FP64, 80 rows, 1555
+// us shared out and 1436 so.
 template <typename T, typename C, int CTAS>
 __global__ void __launch_bounds__(kWalkThreads, CTAS)
-k_observe_walk(const T* __restrict__ fin, int nx, int ny, int rows, Coef<C> k, int mode,
+k_observe_walk(const T* __restrict__ fin, int nx, int ny, int rows, unsigned strips, unsigned items, Coef<C> k, int mode,
                double* __restrict__ rho_o, double* __restrict__ vx_o, double* __restrict__ vy_o,
                VSnap<C>* __restrict__ vsnap, Partial* __restrict__ parts, unsigned* __restrict__ ticket,
                DevStats* __restrict__ ds, const unsigned* __restrict__ status)
 {
     constexpr int NW = kWalkThreads / 32;
     __shared__ WalkPsi<C> sm;
-    __shared__ double red[7 * NW], row_sums[2];
+    __shared__ double red[7 * NW];
     __shared__ unsigned sbad[NW], last;
-    const RowChunk c = row_chunk(blockIdx.y, rows, ny);
-    const int x0 = blockIdx.x * kWalkW, w = min(kWalkW, nx - x0);
-    if (threadIdx.x < 2) row_sums[threadIdx.x] = 0.0;   // (the walk's barriers come before any row's sum)
-    ObsNode<C> node{{mode, nx, ny, rho_o, vx_o, vy_o, (mode & OBS_REDUCE) ? ds : nullptr}, vsnap, row_sums, w, {}};
+    ObsNode<C> node{{mode, nx, ny, rho_o, vx_o, vy_o, (mode & OBS_REDUCE) ? ds : nullptr}, vsnap, {}};
     unsigned bad = 0;
-    tile_walk<T, C>(fin, nx, ny, x0, w, c.y0, c.y1, k, sm, bad, node);
-    if (!(mode & OBS_REDUCE)) return;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        node.acc.row_mid = row_sums[0];
-        node.acc.row0 = row_sums[1];
+    double nodes = 0.0;
+    for (unsigned it = blockIdx.x; it < items; it += gridDim.x) {
+        const RowChunk c = row_chunk(it / strips, rows, ny);
+        const int x0 = int(it % strips) * kWalkW, w = min(kWalkW, nx - x0);
+        tile_walk<T, C>(fin, nx, ny, x0, w, c.y0, c.y1, k, sm, bad, node);
+        nodes += double(c.y1 - c.y0) * double(w);
+        __syncthreads();   // psi of this piece is read
     }
-    reduce_and_fold<C, kWalkThreads>(node.acc, bad, double(c.y1 - c.y0) * double(w), k, nx, red, sbad, &last, parts, ticket,
-                                     ds, status);
+    if (!(mode & OBS_REDUCE)) return;
+    reduce_and_fold<C, kWalkThreads>(node.acc, bad, nodes, k, nx, red, sbad, &last, parts, ticket, ds, status);
 }
 
-template <typename T, typename C, int NT, int NS, int MINB>
+template <typename T, typename C, int NT, int NS, int MINB, bool HALO1>
 int launch_strip(const lbm_params* p, const void* f, int mode, double* rho, double* vx, double* vy, void* vsnap,
            Partial* parts, unsigned* ticket, DevStats* ds, const unsigned* status, cudaStream_t s)
 {
     constexpr size_t smem = strip_smem<T, C, NT, NS>();
     static_assert(smem >= (7 * sizeof(double) + sizeof(unsigned)) * (NT / 32) + sizeof(unsigned), "reduction scratch");
-    auto kern = k_observe_strip<T, C, NT, NS, MINB>;
+    auto kern = k_observe_strip<T, C, NT, NS, MINB, HALO1>;
     static int per_sm = 0, nsm = 0;   // per instantiation (one device per process)
     if (per_sm == 0) {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
@@ -364,32 +373,46 @@ int launch_walk(const lbm_params* p, const void* f, int mode, double* rho, doubl
                 Partial* parts, unsigned* ticket, DevStats* ds, const unsigned* status, int nsm, cudaStream_t s)
 {
     const WalkPlan w = plan_walk(p->nx, p->ny, nsm, CTAS);
-    k_observe_walk<T, C, CTAS><<<dim3(w.sx, w.sy), kWalkThreads, 0, s>>>(
-        (const T*)f, p->nx, p->ny, w.rows, make_coef<C>(*p), mode, rho, vx, vy, (VSnap<C>*)vsnap, parts, ticket, ds, status);
+    const unsigned items = unsigned(w.sx) * unsigned(w.sy);
+    const unsigned grid = w.rows > 64 ? items : std::min(items, unsigned(CTAS * nsm));
+    k_observe_walk<T, C, CTAS><<<grid, kWalkThreads, 0, s>>>(
+        (const T*)f, p->nx, p->ny, w.rows, unsigned(w.sx), items, make_coef<C>(*p), mode, rho, vx, vy, (VSnap<C>*)vsnap, parts, ticket, ds, status);
     return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_E_CUDA;
 }
 
 }  // namespace
 
-// FP32 from 3 * 2^19 nodes (nx % 4 == 0): the strip walk, whose bulk copies
-// keep more of a large lattice in flight; everything else: walks of tiles,
-// which spread over more CTAs and take any width.  lbm_stats, walk of tiles
-// and strip walk: 64 x 64 37 and 72 us (FP64 50 and 370), 512 x 512 50 and 73
-// (FP64 124 and 358), 1024 x 1024 52 and 74 (FP64 353 and 385), 512 x 4096
-// 108 and 76, 1536 x 1536 112 and 80, 4096 x 4096 301 and 188 (FP64 from
-// 1536 x 1536 on within 1 % of each other).  Strips of 512 columns, four CTAs
-// of 128 threads an SM, the left halo's psi off the copying warp: with three
-// lattices in turn and snapshots 75.8 us at 1536 x 1536 and 212.2 at
-// 4096 x 4096; 1024 columns take 89.9 and 224.6, 2048 columns 99.8 and 249.6.
-constexpr long long kObsStripNodes = 3 << 19;
+// FP32 from 3 * 2^20 nodes, where strips of 512 columns idle on at most a
+// third of their columns (nx % 4 == 0): the strip walk, whose bulk copies keep
+// more of a large lattice in flight.  Everything else: walks of tiles, which
+// spread over more CTAs and take any width.  lbm_stats, walk of tiles and
+// strip walk (three lattices in turn; us): 2048 x 1024 64 and 75, 1536 x 1536
+// 76 and 76, 1028 x 2600 77 and 89, 3000 x 1000 79 and 80, 384 x 8192 80 and
+// 78, 768 x 4096 80 and 85, 900 x 4096 93 and 85, 2048 x 2048 102 and 86,
+// 4096 x 4096 322 and 211; by idle columns at 8192 rows, 1000 columns 189 and
+// 125, 768 137 and 123, 640 114 and 124, 560 114 and 124, and 256 x 16384 102
+// and 114.  FP64 walks are 50 us and strips 370 at 64 x 64, 409 and 458 at
+// 1024 x 1024, 1436 and 1679 at 2047 x 2049.  Flat lattices, of one or a few
+// rows and so many columns that every walking CTA would take several pieces
+// of mostly idle warps, keep the strips: 131072 x 1 30 us and 52 (FP64 125 and
+// 171), 400000 x 3 63 and 88 (FP64 697 and 580: only single rows).
+// Strips of 512 columns, four CTAs of 128 threads an SM, the left halo's psi
+// off the copying warp: 75.8 us at 1536 x 1536 and 212.2 at 4096 x 4096;
+// 1024 columns take 89.9 and 224.6, 2048 columns 99.8 and 249.6.
+constexpr long long kObsStripNodes = 3 << 20;
 
 int observe_launch(const lbm_params* p, const void* f, int mode, double* rho, double* vx, double* vy, void* vsnap,
                    Partial* parts, unsigned* ticket, DevStats* ds, const unsigned* status, int nsm, cudaStream_t s)
 {
-    if (p->precision == LBM_FP64)
-        return launch_walk<double, double, 2>(p, f, mode, rho, vx, vy, vsnap, parts, ticket, ds, status, nsm, s);
-    if (lbm_strip_supported(p) && (long long)p->nx * p->ny >= kObsStripNodes)
-        return launch_strip<float, float, 128, 2, 4>(p, f, mode, rho, vx, vy, vsnap, parts, ticket, ds, status, s);
+    const bool fp64 = p->precision == LBM_FP64;
+    if (lbm_strip_supported(p)) {
+        const bool flat = p->ny < (fp64 ? 2 : kWalkH) && (p->nx - 1) / kWalkW >= 2 * kWalkCtas * nsm;
+        if (flat && fp64) return launch_strip<double, double, 64, 4, 2, false>(p, f, mode, rho, vx, vy, vsnap, parts, ticket, ds, status, s);
+        const long long padded = (p->nx + 511LL) / 512 * 512;
+        if (!fp64 && (flat || ((long long)p->nx * p->ny >= kObsStripNodes && 2 * padded <= 3LL * p->nx)))
+            return launch_strip<float, float, 128, 2, 4, true>(p, f, mode, rho, vx, vy, vsnap, parts, ticket, ds, status, s);
+    }
+    if (fp64) return launch_walk<double, double, 2>(p, f, mode, rho, vx, vy, vsnap, parts, ticket, ds, status, nsm, s);
     return launch_walk<float, float, kWalkCtas>(p, f, mode, rho, vx, vy, vsnap, parts, ticket, ds, status, nsm, s);
 }
 
