@@ -265,9 +265,10 @@ int lbm_inject_stage_timeout(lbm_ctx *ctx);
  * strip kernel (nx % 4 == 0).  lbm_set_variant forces one (1 selects the
  * first strip configuration; LBM_E_UNSUPPORTED if the lattice does not
  * allow it); -1 restores the automatic choice: the strip kernel where it
- * applies and is the faster one (FP32 from 2^22 nodes, with the widest strips
- * that cover the width; FP64 from 2^21 nodes) and its strips and row chunks
- * can give every SM a CTA, else the generic kernel.  lbm_autotune picks by
+ * applies and is the faster one (FP32 from 2^22 nodes where strips of 1024 or
+ * 512 columns idle on little of the last one, and flat lattices; FP64 from
+ * 2^21 nodes) and its strips and row chunks can give every SM a CTA, else the
+ * generic kernel.  lbm_autotune picks by
  * timing. */
 int lbm_get_variant(lbm_ctx *ctx, int *variant);
 int lbm_set_variant(lbm_ctx *ctx, int variant);

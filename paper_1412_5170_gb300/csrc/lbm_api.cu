@@ -155,13 +155,22 @@ void launch_generic_scheme(lbm_ctx* c, const void* fin, void* fout)
 // 445); from 2^21 nodes the two are close (1024 x 2560: 867 and 922) and the
 // strip kernel stays the automatic choice where it applies.
 // FP32 below 2^22 nodes: the generic kernel (1536 x 1536 42 us against 68 for
-// 1024-column strips, 512 x 4096 37 and 58).  From there the two-stage carried
-// strips of 1024 or 512 columns, the wider one whose last strip wastes at most
-// a sixteenth of the width: 4096 x 4096 211.5 us with 1024 columns, 252.6
-// with 512 and 252 with the generic kernel; 3072 x 3072 125 and 147 (generic
-// 149); 2560 x 4096 162 and 148 (generic 162).  (2048 columns, 208.5 us at
-// 4096 x 4096, take a whole SM per CTA: three lattices stepping on streams of
-// their own then need 4 % longer than with 1024.)
+// 1024-column strips, 512 x 4096 37 and 58), except on flat lattices, below.
+// From there the cheapest of the carried strips of 1024 columns, those of 512
+// and the generic kernel, each taking a time per column that it covers: 1, 1.09
+// and 1.2, as measured at 3072 and 4096 rows' height (us a step):
+//   width             4096  3840  3456  2888  2564  2432  2304  1800  1712  1536  1280
+//   1024 columns       211   213   214   164   164   161   163   113   113   111   113
+//   512 columns        229   232   207   179   176   150   150   122   121    93    93
+//   generic            252   242   216   188   169   154   152   117   112   102    85
+// so 1024 columns up to a fifth of the strips' columns idle, 512 where these
+// cover better.  (2048 columns, 208.5 us at 4096 x 4096, take a whole SM per
+// CTA: three lattices stepping on streams of their own then need 4 % longer
+// than with 1024.)  Below 9 * 2^19 nodes strips of 512 columns have three
+// stages: 512 x 8192 65.4 us, 71.5 with two, of which more CTAs fit than there
+// are chunks of 16 rows; 512 x 10000 78.7 and 76.4.
+// Flat lattices: walks of 32 x 8 tiles idle on the rows that are not there
+// (1000000 x 2: 117 us, strips 45; 400000 x 3: 48 and 26; 200000 x 7: 32 and 30).
 // Strips also need enough row chunks (at least 16 rows each) to give every SM
 // a CTA.
 int default_config(const lbm_params& p)
@@ -171,15 +180,19 @@ int default_config(const lbm_params& p)
     int cfg = 0;
     if (p.precision == LBM_FP64) {
         if (nodes >= (1 << 21)) cfg = 1;
-    } else if (nodes >= (1 << 22)) {
-        const int n = lbm_strip_config_count(p.precision);
-        for (int threads = 256; threads >= 128 && cfg == 0; threads /= 2) {
-            const long long width = 4LL * threads, padded = (p.nx + width - 1) / width * width;
-            if (16 * padded > 17LL * p.nx) continue;
-            for (int i = 0; i < n; ++i) {   // the last of that shape (256 threads: seam copies one per lane)
-                const StripConfig sc = lbm_strip_config(p.precision, i);
-                if (sc.threads == threads && sc.stages == 2 && sc.warp == 4) cfg = i + 1;
-            }
+    } else if (nodes >= (1 << 22) || p.ny < kWalkH) {
+        int threads = 0, stages = 2;
+        double best = 1.2 * p.nx * (p.ny < kWalkH ? double(kWalkH) / p.ny : 1.0);
+        for (int t = 256; t >= 128; t /= 2) {
+            const long long width = 4LL * t;
+            const double cost = (t == 256 ? 1.0 : 1.09) * double((p.nx + width - 1) / width * width);
+            if (cost <= best) { best = cost; threads = t; }
+        }
+        if (threads == 128 && nodes < (9 << 19)) stages = 3;
+        const int n = threads ? lbm_strip_config_count(p.precision) : 0;
+        for (int i = 0; i < n; ++i) {   // the last carried block strip of that shape
+            const StripConfig sc = lbm_strip_config(p.precision, i);
+            if (sc.threads == threads && sc.stages == stages && sc.warp == (stages == 3 ? 3 : 4)) cfg = i + 1;
         }
     }
     if (cfg == 0) return 0;
