@@ -151,9 +151,12 @@ void launch_generic_scheme(lbm_ctx* c, const void* fin, void* fout)
 }
 
 // Without autotuning.  FP64: the generic kernel, whose tiles keep the FP64
-// pipe busier than the strips' few CTAs (1024 x 1024: 356 us a step against
-// 445); from 2^21 nodes the two are close (1024 x 2560: 867 and 922) and the
-// strip kernel stays the automatic choice where it applies.
+// pipe busier than the strips' few CTAs (1024 x 1024 356 us a step against
+// 445).  From 2^21 nodes the strips stay the automatic choice, as they have
+// been there for callers and for the full-size parity test, not for speed: the
+// generic kernel, which lbm_autotune picks, is 5 to 9 % faster (1024 x 2048
+// 689 and 738, 2048 x 2048 1371 and 1454, 4096 x 4096 5456 and 5721) and more
+// where strips of 256 columns idle (64 x 65536 1371 and 5402).
 // FP32 below 2^22 nodes: the generic kernel (1536 x 1536 42 us against 68 for
 // 1024-column strips, 512 x 4096 37 and 58), except on flat lattices, below.
 // From there the cheapest of the carried strips of 1024 columns, those of 512
