@@ -741,7 +741,7 @@ int build_tiles(lbm_batch* b, const int* host_state)
 // the tail of a run when a few instances remain), the chunks shrink -- down
 // to 16 rows -- so a step is spread over more warps (up to the 14-16 a
 // batched-step SM holds) and its latency (one row walk) shortens.
-int build_items(lbm_batch* b, const int* host_state)
+int build_walk_items(lbm_batch* b, const int* host_state)
 {
     const int nsm = batch_sms();
     long long strip_rows = 0;
@@ -781,7 +781,14 @@ int build_items(lbm_batch* b, const int* host_state)
         B_CUDA(cudaMemcpyAsync(b->items, it.data(), sizeof(BItem) * b->nitems, cudaMemcpyHostToDevice, b->stream));
     B_CUDA(cudaStreamSynchronize(b->stream));
     drop_graphs(b);
-    return build_tiles(b, host_state);
+    return LBM_OK;
+}
+
+// The work items of the running instances for either kind of step.
+int build_items(lbm_batch* b, const int* host_state)
+{
+    const int s = build_walk_items(b, host_state);
+    return s == LBM_OK ? build_tiles(b, host_state) : s;
 }
 
 template <int COLL, int FORC>
@@ -1315,7 +1322,7 @@ int lbm_batch_autotune(lbm_batch* b, int trial_steps, int* columns, int* stages,
             b->ns = cand_ns[ci];
             b->carry = cand_carry[ci];
             b->rows = cand_rows[ri];
-            if ((status = build_items(b, b->h_state)) != LBM_OK) break;
+            if ((status = build_walk_items(b, b->h_state)) != LBM_OK) break;
             // trials read the current state and write the spare buffer only
             const float* fin = b->f[cur0];
             float* fout = b->f[cur0 ^ 1];
