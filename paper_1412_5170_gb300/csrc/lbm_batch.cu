@@ -171,7 +171,7 @@ enum : int { BO_RHO = 1, BO_SNAP = 2, BO_ALL = 4 };
 // that every node is pulled and its psi evaluated once, from one round of
 // loads.  All per-node work is FP32, and maxima are exact in any precision.
 // The sums of drho (mass and probe rows) are FP64: the tile's deviations go to
-// shared memory, one warp adds each column down and then across, 13 FP64
+// shared memory, one warp adds each column down and then across, 12 FP64
 // additions a tile for the mass where shuffle sums in every row's warp took
 // 40.  (With those and the pull repeated after the psi pass lbm_batch_observe
 // took 1.57 ms on the 25 M nodes of 256 sweep instances, with pairs of floats
@@ -270,10 +270,11 @@ k_observe_batch(const float* __restrict__ f, const BInst* __restrict__ inst, con
     if ((t & 31) == 0 && wb) atomicOr(&sbad, wb);
     __syncthreads();
     if (wid > 0) return;
-    double m = 0.0;
+    static_assert(GTY == 8, "column sums as a tree of eight");
+    double c8[GTY];
 #pragma unroll
-    for (int i = 0; i < GTY; ++i) m += double(sd[i][t]);
-    m = warp_sum(m);
+    for (int i = 0; i < GTY; ++i) c8[i] = double(sd[i][t]);
+    const double m = warp_sum(((c8[0] + c8[1]) + (c8[2] + c8[3])) + ((c8[4] + c8[5]) + (c8[6] + c8[7])));
     const bool has_mid = ny / 2 >= y0 && ny / 2 < y0 + h;   // uniform over the CTA
     const double mid = has_mid ? warp_sum(double(sd[ny / 2 - y0][t])) : 0.0;
     const double r0 = y0 == 0 ? warp_sum(double(sd[0][t])) : 0.0;
