@@ -704,7 +704,7 @@ int build_tiles(lbm_batch* b, const int* host_state)
     // separate tiles: two per SM where the batch is that small, 256 nodes at most (smaller ones cost more
     // ring: 146, 163 and 213 us a step at 256, 128 and 64 nodes on 7.5 M nodes).  Walks: chunks of at most
     // 64 rows (25 M nodes: 429 us at 80 rows, 439 at 160, 469 at 320)
-    const int want = (int)std::min<long long>(256, std::max<long long>(32, nodes / (2 * nsm)));
+    const int want = (int)std::min<long long>(kTileNodes, std::max<long long>(32, nodes / (2 * nsm)));
     const int chunk = 8 * (int)std::min<long long>(8, std::max<long long>(1, tiles8 / (16LL * nsm)));
     std::vector<BStepTile> t;
     b->stile_threads = b->tile_walks ? kWalkThreads : 0;

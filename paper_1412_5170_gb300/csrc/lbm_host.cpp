@@ -230,9 +230,9 @@ TilePlan plan_tiles(int nx, int ny, bool fp64, int nsm)
             const int sx = ceil_div(nx, w0), sy = ceil_div(ny, h0);
             if (sy > 65535) continue;
             const int w = ceil_div(nx, sx), h = ceil_div(ny, sy);   // the largest tile
-            if (w * h > 256 || (w + 2) * (h + 2) > 400) continue;
+            if (w * h > kTileNodes || (w + 2) * (h + 2) > kTilePsi) continue;
             const int own = (w * h + 31) / 32, ring = (2 * (w + 2) + 2 * h + 31) / 32;
-            if (32 * (own + ring) > 384) continue;
+            if (32 * (own + ring) > kTileThreads) continue;
             const double tiles = double(sx) * sy, work = own * (psi + col) + ring * psi;
             const double alone = (own + ring + 3) / 4 * psi + (own + 3) / 4 * col;
             const double per_sm = tiles / nsm;

@@ -25,6 +25,7 @@ int lbm_validate_preset(int nx, int ny, int kind, double size, double width, int
 // Tiles of the generic step: the lattice cut into sx x sy nearly equal tiles,
 // one CTA of `threads` threads each.
 struct TilePlan { int sx, sy, threads; };
+constexpr int kTileNodes = 256, kTileThreads = 384, kTilePsi = 400;   // limits of a tile: nodes, threads, psi values
 TilePlan plan_tiles(int nx, int ny, bool fp64, int nsm);
 // Strips of 32 columns and chunks of `rows` rows of the walks of tiles
 // (lbm_tilewalk.cuh), one CTA each, `ctas` of which an SM holds.

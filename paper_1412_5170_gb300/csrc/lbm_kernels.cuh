@@ -9,6 +9,7 @@
 
 #include "lbm.h"
 #include "lbm_device.cuh"
+#include "lbm_host.h"
 #include "lbm_index.cuh"
 
 namespace lbm {
@@ -94,8 +95,6 @@ __device__ __forceinline__ void flag_status(unsigned bad, unsigned* status)
 // ---------------------------------------------------------------------------
 constexpr int GTX = 32, GTY = 8;   // observation tiles
 
-constexpr int kTileNodes = 256, kTileThreads = 384, kTilePsi = 400;
-
 // One tile [x0, x0 + w) x [y0, y0 + h) of an nx x ny lattice: every thread of
 // the CTA calls it, after its griddepcontrol.wait.
 template <typename T, typename C, int COLL, int FORC>
@@ -159,9 +158,7 @@ k_step_generic(const T* fin, T* fout, int nx, int ny, Coef<C> k, unsigned* statu
 }
 
 // ---------------------------------------------------------------------------
-// Observe: rho, v = u + F/(2 rho) at time t for every node, optional FP64
-// field output, optional snapshot compare/store, and one FP64 Partial per
-// block (fixed-order warp-shuffle + shared-memory tree: deterministic).
+// Observation: rho, v = u + F/(2 rho) at time t for every node.
 // ---------------------------------------------------------------------------
 enum : int { OBS_FIELDS = 1, OBS_REDUCE = 2, OBS_SNAP_CMP = 4, OBS_SNAP_STORE = 8 };
 
@@ -215,7 +212,10 @@ template <typename C> __device__ __forceinline__ C obs_huge();
 template <> __device__ __forceinline__ double obs_huge<double>() { return 1e300; }
 template <> __device__ __forceinline__ float obs_huge<float>() { return 1e30f; }
 
-// The per-node work stays in the compute type C: |v|, |v - v_snap| and the
+// Observables of a lattice into one FP64 Partial per 32 x 8 tile (fixed-order
+// warp shuffles and shared memory: deterministic), for callers that bring
+// neither a context nor a workspace (lbm_stats_noalloc).
+// The per-node work stays in the compute type C: |v| and the
 // density extremes (tracked as max drho and max -drho, then rho = rho_ref +
 // drho once per block -- exact, since that sum rounds monotonically in drho)
 // are maxima, which are exact in any precision, so only the mass and the two
@@ -224,13 +224,10 @@ template <> __device__ __forceinline__ float obs_huge<float>() { return 1e30f; }
 // path off the FP64 pipe, which is narrow on this GPU.
 template <typename T, typename C>
 __global__ void __launch_bounds__(GTX * GTY)
-k_observe(const T* __restrict__ fin, int nx, int ny, Coef<C> k, int mode,
-          double* __restrict__ rho_o, double* __restrict__ vx_o, double* __restrict__ vy_o,
-          VSnap<C>* __restrict__ vsnap, Partial* __restrict__ parts, DevStats* __restrict__ ds,
-          const unsigned* __restrict__ status)
+k_observe(const T* __restrict__ fin, int nx, int ny, Coef<C> k, Partial* __restrict__ parts, DevStats* __restrict__ ds)
 {
     __shared__ C sp[(GTY + 2) * (GTX + 2)];
-    __shared__ double red[7][GTX * GTY / 32];
+    __shared__ double red[6][GTX * GTY / 32];
     const int x0 = blockIdx.x * GTX, y0 = blockIdx.y * GTY;
     const size_t n = (size_t)nx * ny;
     unsigned bad = 0;
@@ -245,7 +242,7 @@ k_observe(const T* __restrict__ fin, int nx, int ny, Coef<C> k, int mode,
     const int tx = threadIdx.x % GTX, ty = threadIdx.x / GTX;
     const int x = x0 + tx, y = y0 + ty;
     double mass = 0, rho = 0;
-    C mv = 0, mdv = 0, dmax = -obs_huge<C>(), ndmin = -obs_huge<C>();
+    C mv = 0, dmax = -obs_huge<C>(), ndmin = -obs_huge<C>();
     if (x < nx && y < ny) {
         C g[9];
         pull_node<T, C>(fin, x, y, nx, ny, n, g);
@@ -257,59 +254,43 @@ k_observe(const T* __restrict__ fin, int nx, int ny, Coef<C> k, int mode,
         node_velocity<C>(g, Fx, Fy, k, drho, vx, vy);
         rho = double(k.rho_ref) + double(drho);
         if (!isfinite(drho) || !isfinite(vx) || !isfinite(vy)) bad |= ST_NONFINITE;
-        const size_t o = (size_t)y * nx + x;
-        if (mode & OBS_FIELDS) {
-            if (rho_o) rho_o[o] = rho;
-            if (vx_o) vx_o[o] = double(vx);
-            if (vy_o) vy_o[o] = double(vy);
-        }
-        if (mode & OBS_SNAP_CMP) {
-            const VSnap<C> s = vsnap[o];
-            const C dx = vx - C(s.x), dy = vy - C(s.y);
-            mdv = sqrt(dx * dx + dy * dy);
-            if (isnan(mdv)) mdv = obs_huge<C>();
-        }
-        if (mode & OBS_SNAP_STORE) vsnap[o] = make_vsnap(vx, vy);
         mass = rho;
         mv = sqrt(vx * vx + vy * vy);
         if (isnan(mv)) mv = obs_huge<C>();
         dmax = drho;
         ndmin = -drho;
-        if (ds && x == nx / 2 && y == ny / 2) ds->rho_center = rho;
-        if (ds && x == 0 && y == 0) ds->rho_corner = rho;
+        if (x == nx / 2 && y == ny / 2) ds->rho_center = rho;
+        if (x == 0 && y == 0) ds->rho_corner = rho;
     }
-    if (mode & OBS_REDUCE) {
-        const unsigned allbad = __reduce_or_sync(0xffffffffu, bad);
-        const bool mid_row = y == ny / 2, row_0 = y == 0;      // uniform over the warp
-        double v[7] = {warp_sum(mass), mid_row ? warp_sum(rho) : 0.0, row_0 ? warp_sum(rho) : 0.0,
-                       double(warp_max(mv)), double(warp_max(mdv)), 0.0, 0.0};
-        const C wdmax = warp_max(dmax), wndmin = warp_max(ndmin);
-        v[5] = double(k.rho_ref) + double(wdmax);
-        v[6] = -(double(k.rho_ref) + double(-wndmin));
-        __shared__ unsigned sbad;
-        if (threadIdx.x == 0) sbad = 0;
-        __syncthreads();
-        const int wid = threadIdx.x / 32, lane = threadIdx.x % 32;
-        if (lane == 0) {
+    const unsigned allbad = __reduce_or_sync(0xffffffffu, bad);
+    const bool mid_row = y == ny / 2, row_0 = y == 0;      // uniform over the warp
+    const C wdmax = warp_max(dmax), wndmin = warp_max(ndmin);
+    const double v[6] = {warp_sum(mass), mid_row ? warp_sum(rho) : 0.0, row_0 ? warp_sum(rho) : 0.0, double(warp_max(mv)),
+                         double(k.rho_ref) + double(wdmax), -(double(k.rho_ref) + double(-wndmin))};
+    __shared__ unsigned sbad;
+    if (threadIdx.x == 0) sbad = 0;
+    __syncthreads();
+    const int wid = threadIdx.x / 32, lane = threadIdx.x % 32;
+    if (lane == 0) {
 #pragma unroll
-            for (int j = 0; j < 7; ++j) red[j][wid] = v[j];
-            if (allbad) atomicOr(&sbad, allbad);
+        for (int j = 0; j < 6; ++j) red[j][wid] = v[j];
+        if (allbad) atomicOr(&sbad, allbad);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        constexpr int NW = GTX * GTY / 32;
+        Partial p;
+        p.mass = p.row_mid = p.row0 = 0;
+        p.max_v = p.rho_max = p.neg_rho_min = -1e300;
+        p.max_dv = 0.0;   // (no snapshot to compare with)
+        for (int w = 0; w < NW; ++w) {
+            p.mass += red[0][w]; p.row_mid += red[1][w]; p.row0 += red[2][w];
+            p.max_v = fmax(p.max_v, red[3][w]);
+            p.rho_max = fmax(p.rho_max, red[4][w]); p.neg_rho_min = fmax(p.neg_rho_min, red[5][w]);
         }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            constexpr int NW = GTX * GTY / 32;
-            Partial p;
-            p.mass = p.row_mid = p.row0 = 0;
-            p.max_v = p.max_dv = p.rho_max = p.neg_rho_min = -1e300;
-            for (int w = 0; w < NW; ++w) {
-                p.mass += red[0][w]; p.row_mid += red[1][w]; p.row0 += red[2][w];
-                p.max_v = fmax(p.max_v, red[3][w]); p.max_dv = fmax(p.max_dv, red[4][w]);
-                p.rho_max = fmax(p.rho_max, red[5][w]); p.neg_rho_min = fmax(p.neg_rho_min, red[6][w]);
-            }
-            p.status = sbad | (status ? *status : 0u);
-            p.pad = 0;
-            parts[blockIdx.y * gridDim.x + blockIdx.x] = p;
-        }
+        p.status = sbad;
+        p.pad = 0;
+        parts[blockIdx.y * gridDim.x + blockIdx.x] = p;
     }
 }
 
@@ -406,7 +387,7 @@ __global__ void k_plane_convert(T* __restrict__ fs, double* __restrict__ plane, 
     }
 }
 
-// The observation of a lattice (lbm_observe.cu): mode as k_observe; with
+// The observation of a lattice (lbm_observe.cu): mode of OBS_ flags; with
 // OBS_REDUCE the per-CTA partials (parts, at least as many as 32 x 8 tiles)
 // are reduced in the same launch by the last CTA to finish, in a fixed order,
 // into ds (ticket: a device counter that is 0 between launches).  vsnap holds

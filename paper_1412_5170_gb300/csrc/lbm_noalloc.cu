@@ -105,8 +105,7 @@ template <typename T>
 void launch(const lbm_params& p, const void* f, Partial* parts, DevStats* ds, cudaStream_t s)
 {
     const dim3 grid((p.nx + GTX - 1) / GTX, (p.ny + GTY - 1) / GTY);
-    k_observe<T, T><<<grid, GTX * GTY, 0, s>>>((const T*)f, p.nx, p.ny, make_coef<T>(p), OBS_REDUCE,
-                                               nullptr, nullptr, nullptr, nullptr, parts, ds, nullptr);
+    k_observe<T, T><<<grid, GTX * GTY, 0, s>>>((const T*)f, p.nx, p.ny, make_coef<T>(p), parts, ds);
 }
 
 }  // namespace

@@ -165,12 +165,6 @@ def check(status, what=""):
     return status
 
 
-def strip_observation(p: lbm_params) -> bool:
-    """Whether lbm_stats observes p's lattice in one launch, reduction
-    included: every lattice (walks of tiles down strips of 32 columns)."""
-    return p.nx >= 1 and p.ny >= 1
-
-
 def fma_peak(precision: str = "fp64") -> float:
     """Measured FMA throughput of the current GPU (TFLOP/s) in FP64 or FP32."""
     t = ctypes.c_double()
