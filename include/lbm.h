@@ -472,7 +472,9 @@ int lbm_ws_loss_grad(lbm_ws *w, const float *X_host, const float *Y_host, int n,
 
 /* Adam (beta1 0.9, beta2 0.999, eps 1e-8) on minibatches of the MSE, epochs
  * passes over a per-epoch SplitMix64(seed) shuffle; final_loss (may be NULL)
- * receives the loss over all n samples afterwards. */
+ * receives the loss over all n samples afterwards.  LBM_E_TIMEOUT (a bounded
+ * device-side wait for the weights gave up) leaves the parameters undefined;
+ * lbm_ws_set_params starts over. */
 int lbm_ws_train(lbm_ws *w, const float *X_host, const float *Y_host, int n, int epochs, int batch, float lr,
                  uint64_t seed, float *final_loss);
 
