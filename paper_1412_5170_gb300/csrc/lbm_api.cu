@@ -131,9 +131,10 @@ void launch_generic(lbm_ctx* c, const void* fin, void* fout)
     lc.blockDim = dim3(c->tile.threads);
     // FP64 with more tiles than SMs: a plain launch.  A dependent grid's CTAs
     // take whatever slots the running one leaves, several on one SM while
-    // others stay empty, which costs the FP64 pipe more than the launch gap
-    // (256 x 256: 30.7 us plain, 40.7 us dependent; 64 x 64, one tile per SM:
-    // 10.3 plain, 8.1 dependent).
+    // others stay empty, which can cost the FP64 pipe more than the launch gap
+    // (256 x 256 MRT: 26.7 us plain, 36.0 dependent; BGK, whose tiles are
+    // shorter, 22.6 and 20.9; 64 x 64, one tile per SM: 10.3 plain, 7.3
+    // dependent).
     if (c->p.precision == LBM_FP64 && (long long)c->tile.sx * c->tile.sy > sm_count()) lc.numAttrs = 0;
     cudaLaunchKernelEx(&lc, k_step_generic<T, C, COLL, FORC>, (const T*)fin, (T*)fout, c->p.nx, c->p.ny,
                        make_coef<C>(c->p), c->status);

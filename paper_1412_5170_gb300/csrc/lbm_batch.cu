@@ -174,9 +174,9 @@ enum : int { BO_RHO = 1, BO_SNAP = 2, BO_ALL = 4 };
 // shared memory, one warp adds each column down and then across, 12 FP64
 // additions a tile for the mass where shuffle sums in every row's warp took
 // 40.  (With those and the pull repeated after the psi pass lbm_batch_observe
-// took 1.57 ms on the 25 M nodes of 256 sweep instances, with pairs of floats
-// in place of FP64 sums 0.71, and so no more; the populations' way from HBM is
-// 0.13 of it.)
+// took 1.57 ms on the 25 M nodes of 256 sweep instances, now 0.69, of which the
+// populations' way from HBM is 0.13; sums of float pairs in their place gained
+// nothing.)
 constexpr int kObsThreads = 32 * (GTY + 3);
 __global__ void __launch_bounds__(kObsThreads)
 k_observe_batch(const float* __restrict__ f, const BInst* __restrict__ inst, const BTile* __restrict__ tiles,
@@ -685,8 +685,8 @@ void device_free(void* p) { cudaFree(p); }
 // 3 * 2^20 running nodes or for narrow lattices, walks of tiles from there.
 // Per step, one-warp strip walk / separate tiles / walks of tiles: 24 slabs of
 // 8 x 128 20.6 / 2.5 / 4.7 us, 2.1 M nodes in 64 x 64 lattices 95 / 44 / 43,
-// sweep instances of 3.5 M nodes 88 / 69 / 64, 7.5 M 178 / 146 / 129, 26.6 M
-// 490 / 508 / 429.
+// sweep instances of 3.5 M nodes 88 / 69 / 64, 7.5 M 178 / 146 / 129, 25.0 M
+// 480 / 479 / 398.
 int build_tiles(lbm_batch* b, const int* host_state)
 {
     const int nsm = batch_sms();
@@ -703,7 +703,7 @@ int build_tiles(lbm_batch* b, const int* host_state)
     if (!b->allow_tiles || nodes == 0) return LBM_OK;
     // separate tiles: two per SM where the batch is that small, 256 nodes at most (smaller ones cost more
     // ring: 146, 163 and 213 us a step at 256, 128 and 64 nodes on 7.5 M nodes).  Walks: chunks of at most
-    // 64 rows (25 M nodes: 429 us at 80 rows, 439 at 160, 469 at 320)
+    // 64 rows (25 M nodes: 398 us; with longer ones 429 at 80 rows stood against 439 at 160 and 469 at 320)
     const int want = (int)std::min<long long>(kTileNodes, std::max<long long>(32, nodes / (2 * nsm)));
     const int chunk = 8 * (int)std::min<long long>(8, std::max<long long>(1, tiles8 / (16LL * nsm)));
     std::vector<BStepTile> t;

@@ -8,12 +8,12 @@
 // before.  Each thread loads its nine pulled values of the next tile before
 // it collides the current one, so a CTA always has a tile of loads in flight;
 // a grid of separate tiles (the generic step) waits out the memory latency
-// once per tile instead, at 45 nodes/ns whatever the size.  One barrier per
-// tile: psi is double-buffered.  Per step, separate tiles and this (MRT):
-// 384 x 384 6.0 and 4.6 us, 1023 x 1021 23.1 and 19.5, 2047 x 2049 85.7 and
-// 69.6, 4096 x 4096 335 and 263 (the strip walks 217); 256 sweep instances
-// 508 and 429 (the one-warp strip walk 490).  What bounds it now is issue (55
-// % of the slots at 4096 x 4096) and the latency left per tile; HBM is at 0.67.
+// once per tile instead.  One barrier per tile: psi is double-buffered.  Per
+// step, separate tiles and this (MRT): 384 x 384 6.1 and 4.7 us, 1023 x 1021
+// 22.9 and 19.4, 2047 x 2049 85.4 and 68.8, 4096 x 4096 335 and 252 (the strip
+// walks 211); 256 sweep instances (25 M nodes) 479 and 398 (the one-warp strip
+// walk 480).  What bounds it is issue: 76 to 79 % of the slots at 2047 x 2049,
+// with 467 (MRT) or 525 (BGK) instructions a node.
 #pragma once
 #include <cuda_runtime.h>
 
