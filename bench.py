@@ -48,9 +48,12 @@ TRAFFIC_CAPTURES: dict = {
     ("3b8086d784f35703", 10, 4096): (604.08e6 + 548.31e6),
     ("3b8086d784f35703", 12, 4096): (612.66e6 + 552.19e6),
 }
-# Sources of the block-strip step kernel (its configuration table included).
-KERNEL_SOURCES = ["paper_1412_5170_gb300/csrc/lbm_strip.cuh", "paper_1412_5170_gb300/csrc/lbm_strip_f32.cu",
-                  "paper_1412_5170_gb300/csrc/lbm_device.cuh", "paper_1412_5170_gb300/csrc/lbm_kernels.cuh"]
+# Sources of the single lattice's step kernels: the FP32 strips with their
+# configuration table, the generic tiles and walks with the cuts the planner
+# makes, and the kernel constants.
+KERNEL_SOURCES = ["paper_1412_5170_gb300/csrc/" + f for f in (
+    "lbm_strip.cuh", "lbm_strip_f32.cu", "lbm_warp.cuh", "lbm_async.cuh", "lbm_device.cuh", "lbm_kernels.cuh",
+    "lbm_tilewalk.cuh", "lbm_index.cuh", "lbm_host.h", "lbm_host.cpp")]
 
 
 def kernel_hash() -> str:
@@ -73,8 +76,8 @@ def workload_config(extra=None):
 
 def kernel_name(cfg):
     cid, threads, stages, _ = cfg
-    if cid == 0:
-        return "k_step_generic<float,float,MRT,GUO>"
+    if cid == 0:   # FP32 from 2^17 nodes: walks of tiles
+        return "k_step_walk<MRT,GUO>" if N_SIDE * N_SIDE >= 1 << 17 else "k_step_generic<float,float,MRT,GUO>"
     if threads == 32:
         return "k_step_warp<float,MRT,GUO,%d>" % stages
     return "k_step_strip<float,float,MRT,GUO,%d,%d>" % (threads, stages)
@@ -718,9 +721,10 @@ def _solution(fn, *a):
 # on one launch of the autotuned kernel
 # (sm__sass_thread_inst_executed_op_{dfma,dadd,dmul}_pred_on.sum / nodes),
 # keyed like TRAFFIC_CAPTURES (sha256 of the kernel sources, configuration
-# id, lattice side); unknown otherwise.
+# id, lattice side) and by the SMs of the device, which the tiles are cut for;
+# unknown otherwise.
 FP64_INST_CAPTURES: dict = {
-    ("3b8086d784f35703", 0, 1024): {"dfma": 65036288 / 1048576, "dadd": 77741056 / 1048576,
+    ("3b8086d784f35703", 0, 1024, 152): {"dfma": 65036288 / 1048576, "dadd": 77741056 / 1048576,
                                     "dmul": 34810368 / 1048576},
 }
 
@@ -762,7 +766,7 @@ def run_fp64(args):
         st = lat.stats()
     nodes = side * side
     peak_hbm, kind = measured_peaks()
-    cnt = FP64_INST_CAPTURES.get((kernel_hash(), cfg, side))
+    cnt = FP64_INST_CAPTURES.get((kernel_hash(), cfg, side, torch.cuda.get_device_properties(0).multi_processor_count))
     rate = nodes / (ms * 1e-3)
     if cnt:
         ipn = cnt["dfma"] + cnt["dadd"] + cnt["dmul"]
