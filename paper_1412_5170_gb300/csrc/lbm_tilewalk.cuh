@@ -13,7 +13,7 @@
 // 22.9 and 19.4, 2047 x 2049 85.4 and 68.8, 4096 x 4096 335 and 252 (the strip
 // walks 211); 256 sweep instances (25 M nodes) 479 and 398 (the one-warp strip
 // walk 480).  What bounds it is issue: 76 to 79 % of the slots at 2047 x 2049,
-// with 467 (MRT) or 525 (BGK) instructions a node.
+// with 471 (MRT) or 529 (BGK) instructions a node.
 #pragma once
 #include <cuda_runtime.h>
 
