@@ -495,7 +495,7 @@ __global__ void k_rest_velocity(const BInst* __restrict__ inst, int n_inst, cons
 // Gathered per stored node instead, with a 64-bit division each, the nine
 // products made this FP64-bound (5.6 ms for a sweep of 256 instances, 25 M
 // nodes).  With the fields of preset_density the whole lbm_batch_init of that
-// sweep went from 8.5 to 1.7 ms.
+// sweep went from 8.5 to 1.8 ms.
 __global__ void __launch_bounds__(256)
 k_pops_batch(const BInst* __restrict__ inst, int n_inst, float* __restrict__ f, const double* __restrict__ rho0,
              const Snap* __restrict__ u0, const BGeom* __restrict__ geom)
