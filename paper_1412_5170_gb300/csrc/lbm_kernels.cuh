@@ -185,8 +185,10 @@ __device__ __forceinline__ void node_velocity(const C g[9], C Fx, C Fy, const Co
         vx = fma_rn(0.5f * Fx, inv, jx * inv);
         vy = fma_rn(0.5f * Fy, inv, jy * inv);
     } else {
-        vx = jx / rc + C(0.5) * Fx / rc;
-        vy = jy / rc + C(0.5) * Fy / rc;
+        // one division a component (7.4 FP64 instructions), and where j and F/2
+        // nearly cancel no error of the size of F/2
+        vx = (jx + C(0.5) * Fx) / rc;
+        vy = (jy + C(0.5) * Fy) / rc;
     }
 }
 

@@ -314,9 +314,9 @@ k_observe_strip(const T* __restrict__ fin, int nx, int ny, int nchunks, Coef<C> 
 // 32-column strip's chunk of `rows` rows, shared out over the grid's CTAs, so
 // that a CTA reduces once whatever the lattice's shape.  (With a CTA a piece,
 // wide flat lattices were mostly reductions: lbm_stats at 65536 x 16 took 105
-// us, now 51; 4096 x 256 100, now 51.)  Pieces of more than 64 rows are worth
-// a CTA each, which evens out the last wave: 2047 x 2049 FP64, 80 rows, 1555
-// us shared out and 1436 so.
+// us, now 51; 4096 x 256 100, now 51.)  Pieces of more than 56 rows are worth
+// a CTA each, which evens out the last wave: FP64, 2047 x 2049 (80 rows) 1555
+// us shared out and 1436 so, 2048 x 2048 (64 rows) 1493 and 1457.
 template <typename T, typename C, int CTAS>
 __global__ void __launch_bounds__(kWalkThreads, CTAS)
 k_observe_walk(const T* __restrict__ fin, int nx, int ny, int rows, unsigned strips, unsigned items, Coef<C> k, int mode,
@@ -374,7 +374,7 @@ int launch_walk(const lbm_params* p, const void* f, int mode, double* rho, doubl
 {
     const WalkPlan w = plan_walk(p->nx, p->ny, nsm, CTAS);
     const unsigned items = unsigned(w.sx) * unsigned(w.sy);
-    const unsigned grid = w.rows > 64 ? items : std::min(items, unsigned(CTAS * nsm));
+    const unsigned grid = w.rows > 56 ? items : std::min(items, unsigned(CTAS * nsm));
     k_observe_walk<T, C, CTAS><<<grid, kWalkThreads, 0, s>>>(
         (const T*)f, p->nx, p->ny, w.rows, unsigned(w.sx), items, make_coef<C>(*p), mode, rho, vx, vy, (VSnap<C>*)vsnap, parts, ticket, ds, status);
     return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_E_CUDA;
