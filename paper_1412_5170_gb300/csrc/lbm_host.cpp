@@ -218,7 +218,7 @@ int lbm_validate_preset(int nx, int ny, int kind, double size, double width, int
 // A tenth of the total work is added, so that of two cuts with the same
 // latency the one with less redundant psi wins (streams that share the GPU
 // notice the difference).
-TilePlan plan_tiles(int nx, int ny, bool fp64, int nsm)
+TilePlan plan_tiles(int nx, int ny, bool fp64, int nsm, int max_sy)
 {
     const double psi = fp64 ? 33 : 60, col = fp64 ? 110 : 170;
     const int widths[] = {8, 10, 12, 16, 20, 24, 32, 43, 64};
@@ -228,7 +228,7 @@ TilePlan plan_tiles(int nx, int ny, bool fp64, int nsm)
     for (int w0 : widths)
         for (int h0 : heights) {
             const int sx = ceil_div(nx, w0), sy = ceil_div(ny, h0);
-            if (sy > 65535) continue;
+            if (sy > max_sy) continue;
             const int w = ceil_div(nx, sx), h = ceil_div(ny, sy);   // the largest tile
             if (w * h > kTileNodes || (w + 2) * (h + 2) > kTilePsi) continue;
             const int own = (w * h + 31) / 32, ring = (2 * (w + 2) + 2 * h + 31) / 32;

@@ -26,7 +26,7 @@ int lbm_validate_preset(int nx, int ny, int kind, double size, double width, int
 // one CTA of `threads` threads each.
 struct TilePlan { int sx, sy, threads; };
 constexpr int kTileNodes = 256, kTileThreads = 384, kTilePsi = 400;   // limits of a tile: nodes, threads, psi values
-TilePlan plan_tiles(int nx, int ny, bool fp64, int nsm);
+TilePlan plan_tiles(int nx, int ny, bool fp64, int nsm, int max_sy = 65535);   // (rows of a 2-D grid)
 // Strips of 32 columns and chunks of `rows` rows of the walks of tiles
 // (lbm_tilewalk.cuh), one CTA each, `ctas` of which an SM holds.
 struct WalkPlan { int sx, sy, rows; };

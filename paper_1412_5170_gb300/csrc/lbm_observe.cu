@@ -1,17 +1,19 @@
 // lbm_observe.cu -- the lattice observables (rho, v = u + F/(2 rho) at time t,
 // FP64 mass, max |v|, max |v - v_snap|, density extremes and probes, status)
 // with the walks of the time step -- the strip walk (lbm_strip.cuh) of large
-// FP32 lattices, the walk of tiles (lbm_tilewalk.cuh) of all others: the same row
-// copies or loads, psi and pulled populations, but each node is observed
-// instead of collided, so its populations are read from HBM once (36 B per
-// node in FP32, 72 B in FP64) and nothing is written unless the moment fields
-// or the velocity snapshot are asked for.
+// FP32 lattices, the walk of tiles (lbm_tilewalk.cuh) of all others -- and the
+// moment fields alone on separate tiles: the same row copies or loads, psi and
+// pulled populations, but each node is observed instead of collided, so its
+// populations are read from HBM once (36 B per node in FP32, 72 B in FP64) and
+// nothing is written unless the moment fields or the velocity snapshot are
+// asked for.
 //
 // With OBS_REDUCE every CTA leaves one FP64 Partial, and the last CTA to
 // finish (a ticket counter) reduces all of them in a fixed order into the
 // DevStats record in the same launch: the result is the same bit for bit
 // from run to run.
 #include <algorithm>
+#include <climits>
 #include <cstddef>
 
 #include "lbm.h"
@@ -128,15 +130,15 @@ struct ObsRow {
 // Walk of tiles: one node a thread, a warp one row of the strip.
 template <typename C>
 struct ObsNode {
-    ObsOut to;
+    int mode, nx, ny;
+    DevStats* __restrict__ ds;
     VSnap<C>* __restrict__ vsnap;
     ObsAcc<C, false> acc;
 
     __device__ __forceinline__ void operator()(int y, int x, C (&g)[9], const Stencil<C>& q, const Coef<C>& k,
                                                unsigned& bad)
     {
-        const int mode = to.mode;
-        const size_t o = (size_t)y * to.nx + x;
+        const size_t o = (size_t)y * nx + x;
         VSnap<C> sv{};
         if (mode & OBS_SNAP_CMP) sv = vsnap[o];   // fetched under the node's arithmetic
         C Fx, Fy, d, vx, vy;
@@ -144,18 +146,13 @@ struct ObsNode {
         node_velocity<C>(g, Fx, Fy, k, d, vx, vy);
         acc.node(d, vx, vy);
         if (!isfinite(d) || !isfinite(acc.mv2)) bad |= ST_NONFINITE;
-        const bool mid = y == to.ny / 2;
-        if (mid || y == 0 || (mode & OBS_FIELDS)) {   // (uniform over the warp)
+        const bool mid = y == ny / 2;
+        if (mid || y == 0) {   // (uniform over the warp)
             const double rho = double(k.rho_ref) + double(d);
             if (mid) acc.row_mid += rho;
             if (y == 0) acc.row0 += rho;
-            if (to.ds && mid && x == to.nx / 2) to.ds->rho_center = rho;
-            if (to.ds && y == 0 && x == 0) to.ds->rho_corner = rho;
-            if (mode & OBS_FIELDS) {
-                to.rho_o[o] = rho;
-                to.vx_o[o] = double(vx);
-                to.vy_o[o] = double(vy);
-            }
+            if (mid && x == nx / 2) ds->rho_center = rho;
+            if (y == 0 && x == 0) ds->rho_corner = rho;
         }
         if (mode & OBS_SNAP_CMP) acc.change(vx - C(sv.x), vy - C(sv.y));
         if (mode & OBS_SNAP_STORE) vsnap[o] = make_vsnap(vx, vy);
@@ -315,12 +312,11 @@ k_observe_strip(const T* __restrict__ fin, int nx, int ny, int nchunks, Coef<C> 
 // that a CTA reduces once whatever the lattice's shape.  (With a CTA a piece,
 // wide flat lattices were mostly reductions: lbm_stats at 65536 x 16 took 105
 // us, now 51; 4096 x 256 100, now 51.)  Pieces of more than 56 rows are worth
-// a CTA each, which evens out the last wave: FP64, 2047 x 2049 (80 rows) 1555
-// us shared out and 1436 so, 2048 x 2048 (64 rows) 1493 and 1457.
+// a CTA each, which evens out the last wave: FP64, 2047 x 2049 (80 rows) 1555 us
+// shared out and 1436 so, 2048 x 2048 (64 rows) 1493 and 1457.
 template <typename T, typename C, int CTAS>
 __global__ void __launch_bounds__(kWalkThreads, CTAS)
 k_observe_walk(const T* __restrict__ fin, int nx, int ny, int rows, unsigned strips, unsigned items, Coef<C> k, int mode,
-               double* __restrict__ rho_o, double* __restrict__ vx_o, double* __restrict__ vy_o,
                VSnap<C>* __restrict__ vsnap, Partial* __restrict__ parts, unsigned* __restrict__ ticket,
                DevStats* __restrict__ ds, const unsigned* __restrict__ status)
 {
@@ -328,7 +324,7 @@ k_observe_walk(const T* __restrict__ fin, int nx, int ny, int rows, unsigned str
     __shared__ WalkPsi<C> sm;
     __shared__ double red[7 * NW];
     __shared__ unsigned sbad[NW], last;
-    ObsNode<C> node{{mode, nx, ny, rho_o, vx_o, vy_o, (mode & OBS_REDUCE) ? ds : nullptr}, vsnap, {}};
+    ObsNode<C> node{mode, nx, ny, ds, vsnap, {}};
     unsigned bad = 0;
     double nodes = 0.0;
     for (unsigned it = blockIdx.x; it < items; it += gridDim.x) {
@@ -338,8 +334,80 @@ k_observe_walk(const T* __restrict__ fin, int nx, int ny, int rows, unsigned str
         nodes += double(c.y1 - c.y0) * double(w);
         __syncthreads();   // psi of this piece is read
     }
-    if (!(mode & OBS_REDUCE)) return;
     reduce_and_fold<C, kWalkThreads>(node.acc, bad, nodes, k, nx, red, sbad, &last, parts, ticket, ds, status);
+}
+
+// The tile [x0, x0 + w) x [y0, y0 + h) as step_tile takes it, each node handed to
+// `node` with its pulled populations and the psi stencil around it; every thread
+// of the CTA calls it.  (Sharing this with step_tile through a callable made
+// the step 1 to 2 % slower on small lattices.)
+template <typename T, typename C, class Node>
+__device__ __forceinline__ void tile_nodes(const T* __restrict__ fin, int nx, int ny, int x0, int y0, int w, int h,
+                                           const Coef<C>& k, C* __restrict__ sp, unsigned& bad, Node node)
+{
+    const size_t n = (size_t)nx * ny;
+    const int t = threadIdx.x, W = w + 2;
+    const bool own = t < w * h;
+    int lx, ly;
+    bool live = own;
+    if (own) {
+        ly = t / w;
+        lx = t - ly * w;
+    } else {   // the ring: rows -1 and h (w + 2 nodes each), then columns -1 and w
+        int r = t - (w * h + 31) / 32 * 32;
+        live = r >= 0 && r < 2 * W + 2 * h;
+        if (r < 2 * W) {
+            ly = r < W ? -1 : h;
+            lx = (r < W ? r : r - W) - 1;
+        } else {
+            r -= 2 * W;
+            lx = r < h ? -1 : w;
+            ly = r < h ? r : r - h;
+        }
+    }
+    C g[9];
+    if (live) {
+        const int xs = x0 + lx, ys = y0 + ly;   // one wrap at most: the tile is no larger than the lattice
+        pull_node<T, C>(fin, xs < 0 ? nx - 1 : (xs == nx ? 0 : xs), ys < 0 ? ny - 1 : (ys == ny ? 0 : ys), nx, ny, n, g);
+        sp[(ly + 1) * W + lx + 1] = psi_of_rho<C>(k.rho_ref + sum9(g), k, bad);
+    }
+    __syncthreads();
+    if (own) {
+        const int c = (ly + 1) * W + lx + 1;
+        const Stencil<C> q{sp[c], sp[c + 1], sp[c + W], sp[c - 1], sp[c - W],
+                           sp[c + W + 1], sp[c + W - 1], sp[c - W - 1], sp[c - W + 1]};
+        node(y0 + ly, x0 + lx, g, q);
+    }
+}
+
+// Tile i of sx x sy nearly equal ones, as plan_tiles cuts them.
+struct Tile { int x0, y0, w, h; };
+__device__ __forceinline__ Tile tile_at(unsigned i, int sx, int sy, int nx, int ny)
+{
+    const long long tx = i % unsigned(sx), ty = i / unsigned(sx);
+    const int x0 = int(tx * nx / sx), y0 = int(ty * ny / sy);
+    return Tile{x0, y0, int((tx + 1) * nx / sx) - x0, int((ty + 1) * ny / sy) - y0};
+}
+
+// The moment fields alone, on the generic step's tiles: one round of loads a
+// CTA, whose other CTAs hide it, and no barrier between tiles.
+template <typename T, typename C>
+__global__ void __launch_bounds__(kTileThreads)
+k_moments_tile(const T* __restrict__ fin, int nx, int ny, int sx, int sy, Coef<C> k, double* __restrict__ rho_o,
+               double* __restrict__ vx_o, double* __restrict__ vy_o)
+{
+    __shared__ C sp[kTilePsi];
+    const Tile t = tile_at(blockIdx.x, sx, sy, nx, ny);
+    unsigned bad = 0;   // (no status without a reduction)
+    tile_nodes<T, C>(fin, nx, ny, t.x0, t.y0, t.w, t.h, k, sp, bad, [&](int y, int x, C (&g)[9], const Stencil<C>& q) {
+        C Fx, Fy, d, vx, vy;
+        force<C>(q, k, Fx, Fy);
+        node_velocity<C>(g, Fx, Fy, k, d, vx, vy);
+        const size_t o = (size_t)y * nx + x;
+        rho_o[o] = double(k.rho_ref) + double(d);
+        vx_o[o] = double(vx);
+        vy_o[o] = double(vy);
+    });
 }
 
 template <typename T, typename C, int NT, int NS, int MINB, bool HALO1>
@@ -369,14 +437,23 @@ int launch_strip(const lbm_params* p, const void* f, int mode, double* rho, doub
 }
 
 template <typename T, typename C, int CTAS>
-int launch_walk(const lbm_params* p, const void* f, int mode, double* rho, double* vx, double* vy, void* vsnap,
-                Partial* parts, unsigned* ticket, DevStats* ds, const unsigned* status, int nsm, cudaStream_t s)
+int launch_walk(const lbm_params* p, const void* f, int mode, void* vsnap, Partial* parts, unsigned* ticket, DevStats* ds,
+                const unsigned* status, int nsm, cudaStream_t s)
 {
     const WalkPlan w = plan_walk(p->nx, p->ny, nsm, CTAS);
     const unsigned items = unsigned(w.sx) * unsigned(w.sy);
     const unsigned grid = w.rows > 56 ? items : std::min(items, unsigned(CTAS * nsm));
     k_observe_walk<T, C, CTAS><<<grid, kWalkThreads, 0, s>>>(
-        (const T*)f, p->nx, p->ny, w.rows, unsigned(w.sx), items, make_coef<C>(*p), mode, rho, vx, vy, (VSnap<C>*)vsnap, parts, ticket, ds, status);
+        (const T*)f, p->nx, p->ny, w.rows, unsigned(w.sx), items, make_coef<C>(*p), mode, (VSnap<C>*)vsnap, parts, ticket, ds, status);
+    return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_E_CUDA;
+}
+
+template <typename T, typename C>
+int launch_moments(const lbm_params* p, const void* f, double* rho, double* vx, double* vy, int nsm, cudaStream_t s)
+{
+    const TilePlan t = plan_tiles(p->nx, p->ny, sizeof(C) == sizeof(double), nsm, INT_MAX);
+    k_moments_tile<T, C><<<unsigned(t.sx) * unsigned(t.sy), t.threads, 0, s>>>((const T*)f, p->nx, p->ny, t.sx, t.sy,
+                                                                              make_coef<C>(*p), rho, vx, vy);
     return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_E_CUDA;
 }
 
@@ -391,29 +468,41 @@ int launch_walk(const lbm_params* p, const void* f, int mode, double* rho, doubl
 // 78, 768 x 4096 80 and 85, 900 x 4096 93 and 85, 2048 x 2048 102 and 86,
 // 4096 x 4096 322 and 211; by idle columns at 8192 rows, 1000 columns 189 and
 // 125, 768 137 and 123, 640 114 and 124, 560 114 and 124, and 256 x 16384 102
-// and 114.  FP64 walks are 50 us and strips 370 at 64 x 64, 409 and 458 at
-// 1024 x 1024, 1436 and 1679 at 2047 x 2049.  Flat lattices, of one or a few
-// rows and so many columns that every walking CTA would take several pieces
-// of mostly idle warps, keep the strips: 131072 x 1 30 us and 52 (FP64 125 and
-// 171), 400000 x 3 63 and 88 (FP64 697 and 580: only single rows).
+// and 114.  FP64 lattices walk at any size: 1024 x 1024 322 us, 2048 x 2048 1132,
+// 4096 x 4096 4242 (strips, before one division a velocity component did, 458,
+// 1420 and 5506).  Flat lattices, of one or a few rows and so many columns that
+// every walking CTA would take several pieces of mostly idle warps, keep the
+// strips: 131072 x 1 30 us and 52 (FP64 125 and 171), 400000 x 3 63 and 88 (FP64
+// 697 and 580: only single rows).
 // Strips of 512 columns, four CTAs of 128 threads an SM, the left halo's psi
 // off the copying warp: 75.8 us at 1536 x 1536 and 212.2 at 4096 x 4096;
 // 1024 columns take 89.9 and 224.6, 2048 columns 99.8 and 249.6.
 constexpr long long kObsStripNodes = 3 << 20;
+// The moment fields alone: the generic step's tiles, but FP32 strips from 2^23
+// nodes.  (us, tiles / walk of tiles / strips: 1023 x 1021 33 / 39 / -, 1024 x
+// 1024 33 / 39 / 71, 2048 x 2048 84 / 107 / 90, 33 x 4096 20 / 25 / -, 640 x 8192
+// 102 / 133 / 134, 4096 x 4096 286 / 351 / 255.  FP64, with two divisions a
+// velocity component: 1024 x 1024 316 / 382 / 447, 2048 x 2048 1169 / 1352 / 1418,
+// 33 x 4096 74 / 122 / -, 4096 x 4096 4598 / 5305 / 5413; with one, tiles take 250,
+// 919, 54 and 3602.)
+constexpr long long kMomentStripNodes = 1 << 23;
 
 int observe_launch(const lbm_params* p, const void* f, int mode, double* rho, double* vx, double* vy, void* vsnap,
                    Partial* parts, unsigned* ticket, DevStats* ds, const unsigned* status, int nsm, cudaStream_t s)
 {
-    const bool fp64 = p->precision == LBM_FP64;
-    if (lbm_strip_supported(p)) {
-        const bool flat = p->ny < (fp64 ? 2 : kWalkH) && (p->nx - 1) / kWalkW >= 2 * kWalkCtas * nsm;
-        if (flat && fp64) return launch_strip<double, double, 64, 4, 2, false>(p, f, mode, rho, vx, vy, vsnap, parts, ticket, ds, status, s);
-        const long long padded = (p->nx + 511LL) / 512 * 512;
-        if (!fp64 && (flat || ((long long)p->nx * p->ny >= kObsStripNodes && 2 * padded <= 3LL * p->nx)))
-            return launch_strip<float, float, 128, 2, 4, true>(p, f, mode, rho, vx, vy, vsnap, parts, ticket, ds, status, s);
-    }
-    if (fp64) return launch_walk<double, double, 2>(p, f, mode, rho, vx, vy, vsnap, parts, ticket, ds, status, nsm, s);
-    return launch_walk<float, float, kWalkCtas>(p, f, mode, rho, vx, vy, vsnap, parts, ticket, ds, status, nsm, s);
+    const bool fp64 = p->precision == LBM_FP64, strips = lbm_strip_supported(p);
+    const long long nodes = (long long)p->nx * p->ny, padded = (p->nx + 511LL) / 512 * 512;
+    const bool covered = strips && !fp64 && 2 * padded <= 3LL * p->nx;
+    if (!(mode & OBS_REDUCE) && !(covered && nodes >= kMomentStripNodes))   // the moment fields alone
+        return fp64 ? launch_moments<double, double>(p, f, rho, vx, vy, nsm, s)
+                    : launch_moments<float, float>(p, f, rho, vx, vy, nsm, s);
+    const bool flat = strips && p->ny < (fp64 ? 2 : kWalkH) && (p->nx - 1) / kWalkW >= 2 * kWalkCtas * nsm;
+    if (flat && fp64)
+        return launch_strip<double, double, 64, 4, 2, false>(p, f, mode, rho, vx, vy, vsnap, parts, ticket, ds, status, s);
+    if (!fp64 && (flat || (covered && nodes >= kObsStripNodes)))
+        return launch_strip<float, float, 128, 2, 4, true>(p, f, mode, rho, vx, vy, vsnap, parts, ticket, ds, status, s);
+    if (fp64) return launch_walk<double, double, 2>(p, f, mode, vsnap, parts, ticket, ds, status, nsm, s);
+    return launch_walk<float, float, kWalkCtas>(p, f, mode, vsnap, parts, ticket, ds, status, nsm, s);
 }
 
 }  // namespace lbm
