@@ -45,8 +45,8 @@ SEED = 20141217 + 2 * 1000
 # taken from, the kernel configuration id and the lattice side; when any of
 # them changes the entry no longer matches and traffic is null.
 TRAFFIC_CAPTURES: dict = {
-    ("760dd0d8078eebfc", 10, 4096): (604.21e6 + 548.32e6),
-    ("760dd0d8078eebfc", 12, 4096): (612.19e6 + 552.11e6),
+    ("3970eab011b3729b", 10, 4096): (604.06e6 + 548.37e6),
+    ("3970eab011b3729b", 12, 4096): (612.67e6 + 552.18e6),
 }
 # Sources of the single lattice's step kernels: the FP32 strips with their
 # configuration table, the generic tiles and walks with the cuts the planner
@@ -724,7 +724,7 @@ def _solution(fn, *a):
 # id, lattice side) and by the SMs of the device, which the tiles are cut for;
 # unknown otherwise.
 FP64_INST_CAPTURES: dict = {
-    ("760dd0d8078eebfc", 0, 1024, 152): {"dfma": 65036288 / 1048576, "dadd": 77741056 / 1048576,
+    ("3970eab011b3729b", 0, 1024, 152): {"dfma": 65036288 / 1048576, "dadd": 77741056 / 1048576,
                                     "dmul": 34810368 / 1048576},
 }
 
